@@ -196,9 +196,8 @@ int attention_ctas_per_sm(int head_dim, int group, int batch, bool step,
 cudaError_t configure_attention_instances();
 bool attention_supported(int head_dim, int group);
 // TMA map of one pool [pool_pages][n_kv_heads][page_slots][head_dim] bf16 viewed as
-// {64 elements, head_dim / 64, rows} with a box of {64, head_dim / 64, 16 rows} (half_box:
-// {64, 1, 16 rows}, one 64-column half of a chunk) and the 128-byte swizzle.  Returns a
-// CUresult (0 on success).
+// {64 elements, head_dim / 64, rows} with a box of {64, head_dim / 64, 16 rows} and the 128-byte
+// swizzle.  Returns a CUresult (0 on success).
 // TMA map of a row-major [rows][cols] bf16 matrix with a box of {64 columns, box_rows rows} (128
 // bytes of each row) and the 128-byte swizzle: one K-major operand tile of a tcgen05 product.
 // cols must be a multiple of 8; boxes past the last row or column read zeros.  Returns a CUresult.
@@ -225,14 +224,17 @@ cudaError_t tile_weights(const void *W, int F, int K, void *wt, cudaStream_t str
 cudaError_t launch_gemm_xwt(const CUtensorMap *tw, const void *wt, const CUtensorMap &tx,
                             float *Y, int64_t ldy, int32_t *err, int rows, int F, int K,
                             int splits, bool pdl, cudaStream_t stream);
-// TMA map of a row-major [rows][heads][head_dim] bf16 tensor viewed as {64 elements,
-// head_dim / 64, heads, rows} with a box of {64, 1, box_heads, box_rows} (one 64-column half of
-// box_heads x box_rows head rows) and the 128-byte swizzle.  Boxes past the last row read zeros.
-// Returns a CUresult (0 on success).
+// TMA map of a row-major [rows][heads][head_dim] bf16 tensor viewed as {64 elements, heads, rows,
+// head_dim / 64} with a box of {64, box_heads, box_rows, head_dim / 64} and the 128-byte swizzle:
+// box_rows x box_heads head rows, their 64-column halves one after the other.  Boxes past the last
+// row read zeros.  Returns a CUresult (0 on success).
 int make_rows_tensor_map(CUtensorMap *map, const void *base, int64_t rows, int heads,
                          int head_dim, int box_heads, int box_rows);
-int make_pool_tensor_map(CUtensorMap *map, const void *pool, int64_t rows, int head_dim,
-                         bool half_box);
+int make_pool_tensor_map(CUtensorMap *map, const void *pool, int64_t rows, int head_dim);
+// TMA map of the same pool viewed as {64 elements, 8 rows, head_dim / 64, rows / 8} with a box of
+// {64, 8, head_dim / 64, 2} (a 16-slot chunk: two 8-row groups, each its 64-column halves one after
+// the other) and the 128-byte swizzle.  Returns a CUresult (0 on success).
+int make_pool_group_tensor_map(CUtensorMap *map, const void *pool, int64_t rows, int head_dim);
 cudaError_t launch_append(const AppendView &v, cudaStream_t stream);
 // KV heads per append block (0 if the shape does not fit the append kernel).
 int append_kv_per_block(int n_q_heads, int n_kv_heads, int head_dim);
@@ -317,10 +319,12 @@ struct ham_kv {
   int2 *seg_range = nullptr;
   int4 *prefill_seq = nullptr;     // ham_prefill: per-sequence plan [batch]
   int2 *prefill_rows = nullptr;    // ham_prefill: per-row (position, pool row) [batch * max_slots]
+  int32_t *prefill_next = nullptr; // ham_prefill: the attention's item counter and block count
+  int2 *prefill_order = nullptr;   // ham_prefill: the order of its query blocks
   float *prefill_part = nullptr;   // ham_prefill: split partials (bf16 caches)
   float2 *prefill_part_ml = nullptr;
   int64_t scratch_bytes = 0;
   std::vector<CUtensorMap> tmaps;  // [layers][2]: TMA maps of the K and V pools
-  std::vector<CUtensorMap> tmaps_half;  // [layers][2]: the same, one 64-column half per box
+  std::vector<CUtensorMap> tmaps_group; // [layers][2]: the same by 8-row groups (ham_prefill)
   void *host_stage = nullptr;   // pinned: counters and error word read-back
 };

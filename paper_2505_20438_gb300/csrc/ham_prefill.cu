@@ -20,24 +20,26 @@
 //     lies within ~2^-44 (relative) of a rounding boundary.  This GPU's fp64 pipe would take
 //     about half a millisecond for a 16k-row chunk of a Llama-8B layer; the fp32 pairs take
 //     microseconds.
-//  3. prefill_attn_kernel, one CTA per (KV head, two Q tiles of 128 (query row, head) rows of
-//     one sequence), one CTA an SM: S = Q K^T and O += P V on the 5th-generation tensor cores
-//     (tcgen05.mma kind::f16, M = 128, bf16 operands, fp32 accumulators in tensor memory).
-//     Q, K and V reach shared memory by TMA (64-slot K/V tiles of four 16-slot chunks, each
-//     64-column half one box in the 128-byte swizzle; K and V in rings of their own, filled by
-//     two producer warps whose lanes issue the copies and look the pages up 32 chunks ahead).
-//     Two warps issue the S products of the two Q tiles and two the O products (one thread
-//     issues a tcgen05.mma only about every 125 cycles); eight softmax warps, one thread a row,
+//  3. prefill_attn_kernel, a persistent grid (one CTA an SM) over items of one KV head and two Q
+//     tiles of 128 (query row, head) rows of one sequence: S = Q K^T and O += P V on the
+//     5th-generation tensor cores (tcgen05.mma kind::f16, M = 128, bf16 operands, fp32 accumulators
+//     in tensor memory).  Q, K and V reach shared memory by TMA (128-slot K/V tiles of eight
+//     16-slot chunks, one box each, in one ring; two producer warps look the pages up 32 chunks
+//     ahead).  A warp for each Q tile issues its products; eight softmax warps, one thread a row,
 //     read S from tensor memory, keep the online softmax in fp32 (exp2 domain, running maximum
-//     raised only past 2^8), write the bf16 probabilities to tensor memory columns of their own
-//     (the A operand of O += P V, so the next S is computed meanwhile) and rescale O there when
-//     the maximum moves.  The causal mask applies to the tiles that reach past a row's own slot;
-//     CTAs are scheduled latest query tiles first, the longest rows of the causal triangle.
-//     When the grid would leave SMs idle (a short chunk: few query blocks) it gets a third
-//     dimension, the split over slots: a sequence with L cached slots is cut into up to
-//     floor(L / 512) contiguous ranges of 64-slot tiles (the last range also takes the chunk's
-//     own slots), each CTA streams one range, and a split that is not alone leaves its rows'
-//     unnormalised output, running maximum and sum as a partial.
+//     raised only past 2^8), write the bf16 probabilities over the scores (the A operand of
+//     O += P V) and rescale O in tensor memory when the maximum moves.  The causal mask applies to
+//     the blocks that reach past a row's own slot; items are handed out from a counter in the
+//     plan's order, the longest rows of the causal triangle first.
+//     When the items would leave SMs idle (a short chunk: few query blocks) they are split over
+//     slots: a sequence with L cached slots is cut into up to floor(L / 512) contiguous ranges
+//     of 128-slot tiles (the last range also takes the chunk's own slots), and a split that is
+//     not alone leaves its rows' unnormalised output, running maximum and sum as a partial.
+//     Bound by each Q tile's chain scores -> softmax -> P V -> scores, which the other tile's
+//     covers in part: the tensor pipe is about 60% busy.  4 fresh prompts x 4096 rows of a
+//     Llama-8B layer, the whole call: 492 us, against 565 with 64-slot tiles, four issuing warps whose
+//     operands sat in per-thread registers and a CTA an item; 64 rows over 65,536 slots 93 against
+//     139 us; 4 x 2048 rows over 2048 slots at head_dim 64: 281 against 345.
 //  4. prefill_merge_kernel (split launches only), one warp per (row, head): the split-softmax
 //     merge of the partials in split order (as the decode combine merges its CTAs').
 //
@@ -98,25 +100,41 @@ __device__ __forceinline__ int block_scan(int x, int *red, int *total) {
 __global__ void __launch_bounds__(kPlanThreads) prefill_plan_kernel(PrefillView v, int qb_rows) {
   __shared__ int red[kPlanThreads / 32];
   const int b = blockIdx.x, tid = threadIdx.x, B = v.batch;
-  // The offsets must describe the call's rows: every block checks all of them, so that all
-  // agree, and counts the query blocks of the sequences before its own.
-  int bad_off = 0, qb = 0;
-  for (int i = tid; i < B; i += kPlanThreads) {
-    const int a = v.offsets[i], e = v.offsets[i + 1];
-    bad_off |= e < a;
-    if (i < b && e > a) qb += (e - a + qb_rows - 1) / qb_rows;
-  }
+  if (b == 0 && tid == 0) *v.next_item = 0;  // the attention's items are handed out from here
+  // The offsets must describe the call's rows: every block checks all of them, so that all agree.
+  int bad_off = 0;
+  for (int i = tid; i < B; i += kPlanThreads) bad_off |= v.offsets[i + 1] < v.offsets[i];
   if (tid == 0) bad_off |= v.offsets[0] != 0 || v.offsets[B] != v.rows;
   bad_off = __syncthreads_or(bad_off);
-  qb = block_sum(qb, red);
   if (bad_off) {
     if (tid == 0) {
       v.seq_info[b] = make_int4(-1, 0, 0, 0);
-      if (b == 0) record_error(v.err, HAM_DEVERR_NTOK);
+      if (b == 0) {
+        v.next_item[1] = 0;  // no query blocks
+        record_error(v.err, HAM_DEVERR_NTOK);
+      }
     }
     return;
   }
   const int a = v.offsets[b], n = v.offsets[b + 1] - a;
+  // The order of the query blocks in the attention: later blocks of the chunks (longer rows of the
+  // causal triangle) first, sequence by sequence.  Block j comes after all blocks j' > j and the
+  // blocks j of earlier sequences.
+  auto blocks_of = [&](int c) { return (v.offsets[c + 1] - v.offsets[c] + qb_rows - 1) / qb_rows; };
+  for (int j = tid; j < blocks_of(b); j += kPlanThreads) {
+    int at = 0;
+    for (int c = 0; c < B; ++c) {
+      const int m = blocks_of(c);
+      at += max(0, m - 1 - j) + (c < b && m > j ? 1 : 0);
+    }
+    v.order[at] = make_int2(b, j);
+  }
+  if (b == 0) {
+    int m = 0;
+    for (int c = tid; c < B; c += kPlanThreads) m += blocks_of(c);
+    m = block_sum(m, red);
+    if (tid == 0) v.next_item[1] = m;
+  }
   const int L = v.num_slots[b];
   int err = 0;
   if (L < 0 || L > v.max_slots) err = HAM_DEVERR_SLOTS;
@@ -139,7 +157,7 @@ __global__ void __launch_bounds__(kPlanThreads) prefill_plan_kernel(PrefillView 
     for (int j = tid; j < n; j += kPlanThreads) v.row_info[a + j] = make_int2(0, -1);
     if (tid == 0) {
       record_error(v.err, err);
-      v.seq_info[b] = make_int4(-1, n, qb, 1);
+      v.seq_info[b] = make_int4(-1, n, 0, 1);
     }
     return;
   }
@@ -176,7 +194,7 @@ __global__ void __launch_bounds__(kPlanThreads) prefill_plan_kernel(PrefillView 
     carry += total;
   }
   if (tid == 0) {
-    v.seq_info[b] = make_int4(L, n, qb, 1);
+    v.seq_info[b] = make_int4(L, n, 0, 1);
     v.num_slots[b] = L + n;
     v.num_tokens[b] = t0 + carry;
   }
@@ -371,44 +389,83 @@ __global__ void __launch_bounds__(kRopeThreads) prefill_rope_kernel(PrefillView 
 // ------------------------------------------------------------------------------------
 // 3. causal attention of the chunk, on the 5th-generation tensor cores (tcgen05)
 // ------------------------------------------------------------------------------------
-// A CTA covers one KV head and two Q tiles of 128 rows each; a row is a (query row, head)
-// pair, m = (row - first row of the tile) * G + head within the group, and sits in TMEM lane m.
-// Tensor-memory columns per Q tile q: S_q (64 fp32 scores of the current 64-slot K tile), P_q
-// (the bf16 probabilities of the tile as pairs: the A operand of O += P V) and O_q (head_dim
-// fp32).  The products of a Q tile are issued by two warps, one for S = Q K^T and one for
-// O += P V: one thread issues a tcgen05.mma only about every 125 cycles (measured on GB300),
-// so a single issuer would keep the tensor cores half idle.  Because P has columns of its own,
-// S_q(t + 1) is computed while the softmax group still works on tile t.
+// A work item is one KV head, two Q tiles of 128 rows each and (split launches) one range of
+// slots; a row is a (query row, head) pair, m = (row - first row of the tile) * G + head within
+// the group, and sits in TMEM lane m.  CTAs (one an SM) take items from a counter, the longest
+// rows of the causal triangle first; an item's last softmax and output run beside the next one's
+// first copies.
+//
+// K and V come in tiles of 128 slots; the softmax works on blocks of 64 (half tiles).  Tensor-memory
+// columns per Q tile q: two blocks of scores S_q (64 fp32 each; the first 32 columns of a block then
+// hold its probabilities P, bf16 pairs, the A operand of O += P V) and O_q (head_dim fp32).  One
+// thread a Q tile issues its products: O += P V of a block, then the S whose columns that frees.
+// Products execute in issue order, so S overwrites P only after P V has read it.
+//  - head_dim 128: S of a tile (N = 128) follows P V of the second block of the tile before.  While
+//    the products of one Q tile run, the other's softmax does: the two softmax groups take turns,
+//    tile by tile.  (Left to themselves they fall into step, compete for the issue slots and then
+//    for the tensor cores: 6% slower.  With S in blocks, N = 64, a product takes the 64 cycles of
+//    N = 128, bound by the shared-memory reads of Q: also slower.)
+//  - head_dim 64: half the products for the same softmax, which bounds it: S of a block (N = 64) is
+//    two blocks ahead and the softmax never waits (13% faster than S of whole tiles).
+// Why blocks: the hot code of the warps together has to stay in the instruction cache.  With a row
+// of 128 scores unrolled it was about 26 KB, and a tile's softmax took 1.7 times as long as in a
+// kernel of its own.
 template <int D>
 struct TcShape {
-  static constexpr int kTile = 64;                           // slots per K/V tile
+  static constexpr int kTile = 128;                          // slots per K/V tile
   static constexpr int kChunks = kTile / kChunkSlots;        // 16-slot TMA chunks per tile
+  static constexpr int kBlock = 64;                          // slots per softmax block
+  static constexpr int kBlockChunks = kBlock / kChunkSlots;
+  static constexpr bool kTileS = D == 128;                   // S by tiles; else by blocks, two ahead
+  static constexpr int kSSlots = kTileS ? kTile : kBlock;    // slots (N) of an S product
   static constexpr int kHalves = D / 64;                     // 64-column halves of a row
-  static constexpr int kHalfTileBytes = kTile * 128;         // one half of a K or V tile
-  static constexpr int kKVBytes = kHalves * kHalfTileBytes;  // a K (or V) tile
-  static constexpr int kKStages = D == 128 ? 4 : 8;          // K tiles in flight
-  static constexpr int kVStages = D == 128 ? 5 : 8;          // V tiles in flight
+  // A K (or V) tile, a ring stage: 8-row groups, each its 64-column halves one after the other
+  // (8 rows of 128 bytes in the 128-byte swizzle), so that a 16-slot chunk is one TMA box.
+  static constexpr int kGroupBytes = kHalves * 1024;
+  static constexpr int kChunkBytes = 2 * kGroupBytes;
+  static constexpr int kKVBytes = kChunks * kChunkBytes;
+  static constexpr int kStages = D == 128 ? 5 : 10;          // K and V tiles in flight
   static constexpr int kQHalfBytes = 128 * 128;              // one half of a Q tile
   static constexpr int kQBytes = kHalves * kQHalfBytes;
-  static constexpr int kOffK = 2 * kQBytes;                  // Q tiles at 0
-  static constexpr int kOffV = kOffK + kKStages * kKVBytes;
-  static constexpr int kOffBar = kOffV + kVStages * kKVBytes;
-  // k_full, k_empty [kKStages]; v_full, v_empty [kVStages]; q_full; s_full, s_free, p_full,
-  // pv_done [2]; mma_done
-  static constexpr int kBars = 2 * kKStages + 2 * kVStages + 10;
-  static constexpr int kSmem = 1024 + kOffBar + kBars * 8 + 16;
+  static constexpr int kOffRing = 2 * kQBytes;               // Q tiles at 0
+  static constexpr int kOffBar = kOffRing + kStages * kKVBytes;
+  // full, empty [kStages]; q_full, q_empty, o_full, pv_done [2]; s_full, p_full [2][2];
+  // item_full, item_empty [kItems]; mma_done; turn [2]
+  static constexpr int kItems = 4;                           // items handed out ahead
+  static constexpr int kBars = 2 * kStages + 19 + 2 * kItems;
+  static constexpr int kOffItems = kOffBar + (kBars * 8 + 15) / 16 * 16;
+  static constexpr int kOffMisc = kOffItems + kItems * (int)sizeof(PrefillItem);
+  static constexpr int kSmem = 1024 + kOffMisc + 16;
   static constexpr uint32_t kTmemCols = 512;
-  static constexpr int kOffP = 2 * kTile;                    // TMEM column of P_0 (S_0 at 0)
-  static constexpr int kOffO = kOffP + kTile;                // TMEM column of O_0
-  // softmax: warps 0-3 (Q tile 0) and 4-7 (Q tile 1); TMA producers of Q and K (8) and of V
-  // (10); MMA issue of S_0 (9), S_1 (11), O_0 (12), O_1 (13).
-  static constexpr int kProducerWarp = 8, kVProducerWarp = 10;
-  static constexpr int kSWarp0 = 9, kSWarp1 = 11, kOWarp0 = 12, kOWarp1 = 13;
-  static constexpr int kThreads = 14 * 32;
+  static constexpr int kOffO = 2 * kTile;                    // TMEM column of O_0 (S_0 at 0)
+  // softmax: warps 0-3 (Q tile 0) and 4-7 (Q tile 1); TMA producers of K (8) and of Q and V (9,
+  // which also fetches the items); the MMA issuers of Q tile 0 (10) and 1 (11).
+  static constexpr int kProducerWarp = 8, kVProducerWarp = 9, kMmaWarp = 10;
+  static constexpr int kThreads = 12 * 32;
   static_assert(D == 64 || D == 128, "head_dim 64 or 128");
   static_assert(kOffO + 2 * D <= (int)kTmemCols, "TMEM columns");
   static_assert(kSmem <= 227 * 1024, "shared memory");
 };
+
+// Scores of the slots past `seen` (of a block's 64) become -inf: the causal edge, the chunk's end.
+__device__ __forceinline__ void mask_scores(uint32_t (&r)[2][32], int seen) {
+#pragma unroll
+  for (int x = 0; x < 2; ++x)
+#pragma unroll
+    for (int c = 0; c < 32; ++c)
+      if (32 * x + c > seen) r[x][c] = 0xFF800000u;
+}
+__device__ __forceinline__ float max_score(const uint32_t (&r)[2][32]) {
+  float m[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+  for (int c = 0; c < 32; c += 4)
+#pragma unroll
+    for (int x = 0; x < 2; ++x) {
+      m[2 * x] = fmaxf(fmaxf(m[2 * x], __uint_as_float(r[x][c])), __uint_as_float(r[x][c + 1]));
+      m[2 * x + 1] = fmaxf(fmaxf(m[2 * x + 1], __uint_as_float(r[x][c + 2])), __uint_as_float(r[x][c + 3]));
+    }
+  return fmaxf(fmaxf(m[0], m[1]), fmaxf(m[2], m[3]));
+}
 
 template <typename OutT>
 __device__ __forceinline__ void store_row32(OutT *dst, const uint32_t (&o)[32], float scale) {
@@ -429,6 +486,42 @@ __device__ __forceinline__ void store_row32(OutT *dst, const uint32_t (&o)[32], 
   }
 }
 
+// Items of a launch: every (KV head, query block, split), KV head fastest, the query blocks in the
+// plan's order.  False: the sequence was refused, or has fewer splits.
+__device__ __forceinline__ bool decode_item(const PrefillView &v, int id, int nblocks, int tile,
+                                            PrefillItem &it) {
+  const int Hkv = v.n_kv_heads, R = 128 / (v.n_q_heads / Hkv);
+  const int rest = id / Hkv, z = rest / nblocks;
+  const int2 blk = v.order[rest - z * nblocks];  // (sequence, query block of its chunk)
+  const int4 si = v.seq_info[blk.x];
+  const int L = si.x, n = si.y, qb0 = blk.y * 2 * R;
+  const int zs = prefill_splits(L, v.splits);
+  if (L < 0 || z >= zs) return false;
+  // Split z of the sequence's zs takes tiles t0 .. t1 - 1: the cached part's whole tiles cut
+  // evenly, the last split also the rest (the chunk's own slots, the causal edge).  Every split
+  // starts at or before slot L - tile, which every row attends, so no row of a split is empty.
+  const int rows_q0 = min(R, n - qb0), rows_q1 = max(0, min(R, n - qb0 - R));
+  const int end0 = L + qb0 + rows_q0, end1 = rows_q1 > 0 ? end0 + rows_q1 : 0;
+  const int n0 = (end0 + tile - 1) / tile, n1 = (end1 + tile - 1) / tile;
+  const int ntiles = max(n0, n1), Lt = L / tile;  // (Lt * zs: below 2^31 / 128 * 32)
+  const int t0 = z * Lt / zs, t1 = z + 1 == zs ? ntiles : (z + 1) * Lt / zs;
+  it.valid = 1;
+  it.b = blk.x;
+  it.g = id - rest * Hkv;
+  it.L = L;
+  it.n = n;
+  it.qb0 = qb0;
+  it.row0 = v.offsets[blk.x];
+  it.z = z;
+  it.zs = zs;
+  it.t0 = t0;
+  it.nt0 = max(0, min(t1, n0) - t0);
+  it.nt1 = max(0, min(t1, n1) - t0);
+  it.end0 = end0;
+  it.end1 = end1;
+  return true;
+}
+
 // One CTA per SM (shared memory and 512 TMEM columns).
 template <int D, typename OutT>
 __global__ void __launch_bounds__(TcShape<D>::kThreads, 1)
@@ -436,66 +529,42 @@ __global__ void __launch_bounds__(TcShape<D>::kThreads, 1)
                         const __grid_constant__ CUtensorMap tmap_k,
                         const __grid_constant__ CUtensorMap tmap_v, const PrefillView v) {
   using S = TcShape<D>;
-  const int Hq = v.n_q_heads, Hkv = v.n_kv_heads, G = Hq / Hkv, R = 128 / G, QB = 2 * R;
-  const int g = blockIdx.x;
-  const int64_t xq = (int64_t)gridDim.y - 1 - blockIdx.y;  // latest query blocks first
-  int lo = 0, hi = v.batch - 1;                            // the sequence of query block xq
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (v.seq_info[mid].z <= xq) lo = mid; else hi = mid - 1;
-  }
-  const int4 si = v.seq_info[lo];
-  if (si.x < 0 || xq < si.z || xq >= (int64_t)si.z + (si.y + QB - 1) / QB) return;
-  const int b = lo, L = si.x, n = si.y;
-  const int qb0 = (int)(xq - si.z) * QB;
-  const int64_t row0 = v.offsets[b];
-  // rows of each Q tile and the K/V tiles they reach (slots 0 .. L + last row)
-  const int rows_q0 = min(R, n - qb0), rows_q1 = max(0, min(R, n - qb0 - R));
-  int ntile[2];
-  ntile[0] = (L + qb0 + rows_q0 + S::kTile - 1) / S::kTile;
-  ntile[1] = rows_q1 > 0 ? (L + qb0 + R + rows_q1 + S::kTile - 1) / S::kTile : 0;
-  const int ntiles = max(ntile[0], ntile[1]);
-  const int kv_end = L + qb0 + (rows_q1 > 0 ? R + rows_q1 : rows_q0);  // no slot >= is attended
-  // Split z of the sequence's zs takes tiles t0 .. t1 - 1: the cached part's whole tiles cut
-  // evenly, the last split also the rest (the chunk's own slots, the causal edge).  Every split
-  // starts at or before slot L - 64, which every row attends, so no row of a split is empty.
-  const int zs = prefill_splits(L, (int)gridDim.z), z = (int)blockIdx.z;
-  if (z >= zs) return;
-  const int Lt = L / S::kTile;
-  const int t0 = (int)((int64_t)z * Lt / zs);
-  const int t1 = z + 1 == zs ? ntiles : (int)((int64_t)(z + 1) * Lt / zs);
-  const int ntq[2] = {max(0, min(t1, ntile[0]) - t0), max(0, min(t1, ntile[1]) - t0)};
-  const int nts = max(ntq[0], ntq[1]);  // tiles this CTA streams
-
+  const int Hq = v.n_q_heads, Hkv = v.n_kv_heads, G = Hq / Hkv, R = 128 / G;
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = reinterpret_cast<uint8_t *>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  uint64_t *k_full = reinterpret_cast<uint64_t *>(smem + S::kOffBar);
-  uint64_t *k_empty = k_full + S::kKStages, *v_full = k_empty + S::kKStages;
-  uint64_t *v_empty = v_full + S::kVStages, *q_full = v_empty + S::kVStages;
-  uint64_t *s_full = q_full + 1, *s_free = q_full + 3, *p_full = q_full + 5;
-  uint64_t *pv_done = q_full + 7, *mma_done = q_full + 9;
-  uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(k_full + S::kBars);
+  uint64_t *full = reinterpret_cast<uint64_t *>(smem + S::kOffBar);
+  uint64_t *empty = full + S::kStages, *q_full = empty + S::kStages, *q_empty = q_full + 2;
+  uint64_t *o_full = q_full + 4, *pv_done = q_full + 6, *s_full = q_full + 8, *p_full = q_full + 12;
+  uint64_t *item_full = q_full + 16, *item_empty = item_full + S::kItems;
+  uint64_t *mma_done = item_empty + S::kItems, *turn = mma_done + 1;
+  PrefillItem *items = reinterpret_cast<PrefillItem *>(smem + S::kOffItems);
+  uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(smem + S::kOffMisc);
   volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = __shfl_sync(kFull, tid >> 5, 0), lane = tid & 31;
   if (tid == 0) {
-    // a stage is free once the products of both Q tiles that read it have completed
-    for (int s = 0; s < S::kKStages; ++s) {
-      mbar_init(&k_full[s], 1);
-      mbar_init(&k_empty[s], 2);
+    // a stage is free once the products of both Q tiles that read it completed
+    for (int s = 0; s < S::kStages; ++s) {
+      mbar_init(&full[s], 1);
+      mbar_init(&empty[s], 2);
     }
-    for (int s = 0; s < S::kVStages; ++s) {
-      mbar_init(&v_full[s], 1);
-      mbar_init(&v_empty[s], 2);
-    }
-    mbar_init(q_full, 1);
     for (int q = 0; q < 2; ++q) {
-      mbar_init(&s_full[q], 1);
-      mbar_init(&s_free[q], 4);  // the softmax group has read S_q (one arrival per warp)
-      mbar_init(&p_full[q], 4);  // ... and written P_q
+      mbar_init(&q_full[q], 1);
+      mbar_init(&q_empty[q], 1);
+      mbar_init(&o_full[q], 1);
       mbar_init(&pv_done[q], 1);
+      for (int x = 2 * q; x < 2 * q + 2; ++x) {
+        mbar_init(&s_full[x], 1);
+        mbar_init(&p_full[x], 4);  // the softmax group has written a block's P (one arrival per warp)
+      }
     }
-    mbar_init(mma_done, 4);      // the four MMA warps
+    for (int x = 0; x < S::kItems; ++x) {
+      mbar_init(&item_full[x], 1);
+      mbar_init(&item_empty[x], 11);     // 8 softmax warps, the K producer, 2 MMA warps
+    }
+    mbar_init(mma_done, 2);
+    mbar_init(&turn[0], 4);  // the turn of Q tile 0's / 1's softmax group (one arrival per warp)
+    mbar_init(&turn[1], 4);
     *abort_flag = 0;
     fence_mbar_init();
   }
@@ -504,331 +573,436 @@ __global__ void __launch_bounds__(TcShape<D>::kThreads, 1)
     prefetch_tensormap(&tmap_k);
     prefetch_tensormap(&tmap_v);
   }
-  if (warp == S::kSWarp0) tmem_alloc<S::kTmemCols>(tmem_slot);
+  if (warp == S::kMmaWarp) tmem_alloc<S::kTmemCols>(tmem_slot);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
-  // ring and data waits: the launch's limit; draining in-flight work keeps the default 2 s
+  // ring and data waits: the launch's limit; item hand-over and the draining of in-flight work
+  // keep the default 2 s
   const uint64_t wait_lim = data_wait_limit(v.wait_ns);
-
-  if (warp == S::kProducerWarp || warp == S::kVProducerWarp) {
-    // ------------------------------------------------------------ producers: TMA copies
-    // One warp streams Q and the K tiles, another the V tiles, each as far ahead as its ring
-    // allows (K tiles are needed a tile before V tiles and are released earlier).  A chunk at or
-    // past kv_end is not copied: its rows are masked (K) or zeroed (V).
-    const bool is_v = warp == S::kVProducerWarp;
-    const uint64_t pol_kv = policy_evict_last();   // every query block of the sequence reads them
-    if (!is_v && lane == 0) {
-      const uint64_t pol_q = policy_evict_first();
-      const int nq = rows_q1 > 0 ? 2 : 1;
-      mbar_arrive_tx(q_full, (uint32_t)(nq * S::kQBytes));
-      for (int q = 0; q < nq; ++q)
-        for (int hh = 0; hh < S::kHalves; ++hh)
-          tma_load_4d(smem + q * S::kQBytes + hh * S::kQHalfBytes, &tmap_q, 0, hh, g * G,
-                      (int)(row0 + qb0 + q * R), q_full, pol_q);
-    }
-    const int stages = is_v ? S::kVStages : S::kKStages;
-    uint8_t *ring = smem + (is_v ? S::kOffV : S::kOffK);
-    uint64_t *full = is_v ? v_full : k_full, *empty = is_v ? v_empty : k_empty;
-    const CUtensorMap *map = is_v ? &tmap_v : &tmap_k;
-    // Page-table entries of 32 chunks (4 tiles) at a time, one per lane, requested a batch
-    // ahead: lane l holds the pool row of chunk base + l (-1: at or past kv_end; -2: a page
-    // outside the pool).
-    const int nchunks = (kv_end + kChunkSlots - 1) / kChunkSlots;
-    auto lookup = [&](int base) {
-      int row = -1;
-      if (base + lane < nchunks) {
-        const int slot0 = (base + lane) * kChunkSlots;
-        const int page = v.page_table[(int64_t)b * v.max_pages + slot0 / v.page_slots];
-        row = page < 0 || page >= v.pool_pages
-                  ? -2
-                  : (int)(((int64_t)page * Hkv + g) * v.page_slots + slot0 % v.page_slots);
-      }
-      return row;
-    };
-    constexpr int kTilesPerBatch = 32 / S::kChunks;
-    const int cbase = t0 * S::kChunks;  // the split's first chunk
-    int row = lookup(cbase), row_next = lookup(cbase + 32);
-    int issued = 0;
-    for (int i = 0; i < nts; ++i) {  // tile t0 + i, the i-th of this CTA's ring
-      if (i > 0 && i % kTilesPerBatch == 0) {
-        row = row_next;
-        row_next = lookup(cbase + (i / kTilesPerBatch + 1) * 32);
-      }
-      int my_row = __shfl_sync(kFull, row, ((i % kTilesPerBatch) * S::kChunks + lane) & 31);
-      if (lane >= S::kChunks) my_row = -1;
-      if (__any_sync(kFull, my_row == -2)) {  // the plan validated the table: this ends the CTA
-        if (lane == 0) {
-          record_error(v.err, HAM_DEVERR_PAGE);
-          *abort_flag = 1;
-        }
-        break;
-      }
-      const int st = i % stages;
-      int ok_wait = 1;
-      if (lane == 0 && i >= stages)
-        ok_wait = thread_wait(&empty[st], (uint32_t)((i / stages) - 1) & 1u, abort_flag, true,
-                              wait_lim);
-      if (!__shfl_sync(kFull, ok_wait, 0)) {
-        if (lane == 0 && !*abort_flag) {
-          record_error(v.err, HAM_DEVERR_TIMEOUT);
-          *abort_flag = 1;
-        }
-        break;
-      }
-      // lane 0 posts the byte count, then lane c issues chunk c's boxes, so that the warp has
-      // the tile's copies in flight at once
-      const uint32_t nck = __popc(__ballot_sync(kFull, my_row >= 0));
-      if (lane == 0) mbar_arrive_tx(&full[st], nck * (uint32_t)(kChunkSlots * D * 2));
-      __syncwarp();
-      if (my_row >= 0) {
-#pragma unroll
-        for (int hh = 0; hh < S::kHalves; ++hh)
-          tma_load_3d(ring + st * S::kKVBytes + hh * S::kHalfTileBytes + lane * kChunkSlots * 128,
-                      map, 0, hh, my_row, &full[st], pol_kv);
-      }
-      issued = i + 1;
-    }
-    if (lane == 0) {
-      // every copy this warp issued lands before the CTA can exit
-      if (!is_v) thread_wait(q_full, 0u, abort_flag, false);
-      for (int t = max(0, issued - stages); t < issued; ++t)
-        thread_wait(&full[t % stages], (uint32_t)(t / stages) & 1u, abort_flag, false);
-    }
-  } else if (warp == S::kSWarp0 || warp == S::kSWarp1 || warp == S::kOWarp0 ||
-             warp == S::kOWarp1) {
-    // ------------------------------------------------------------ MMA issue (lane 0)
-    // S warp of Q tile q: S_q(t) = Q_q K_t^T once the softmax group has read S_q(t - 1) into
-    // registers (s_free) and K_t has landed.  O warp: O_q += P_q(t) V_t once the group has
-    // written P_q(t) (p_full) and V_t has landed; the group waits for pv_done before it writes
-    // the next P or rescales O.  A K or V stage is released by a commit for each Q tile that
-    // reads it; a tile that only one Q tile reaches is released twice by that tile's warp.
-    const bool is_o = warp == S::kOWarp0 || warp == S::kOWarp1;
-    const int q = (warp == S::kSWarp0 || warp == S::kOWarp0) ? 0 : 1;
-    const int nt = ntq[q], other = ntile[q ^ 1];  // (tile t0 + i; other: absolute)
-    bool ok = true;
-    if (!is_o) {
-      constexpr uint32_t id_s = idesc_bf16(128, S::kTile, false);  // K-major Q and K
-      const uint32_t q_base = smem_u32(smem) + q * S::kQBytes;
-      if (nt > 0) ok = warp_wait(q_full, 0u, abort_flag, wait_lim);
-      for (int i = 0; ok && i < nt; ++i) {
-        const int t = t0 + i, ks = i % S::kKStages;
-        if ((i > 0 && !warp_wait(&s_free[q], (uint32_t)(i - 1) & 1u, abort_flag, wait_lim)) ||
-            !warp_wait(&k_full[ks], (uint32_t)(i / S::kKStages) & 1u, abort_flag, wait_lim)) {
-          ok = false;
-          break;
-        }
-        if (lane == 0) {
-          tc_fence_after();
-          const uint32_t kt = smem_u32(smem + S::kOffK + ks * S::kKVBytes);
-#pragma unroll
-          for (int k = 0; k < D / 16; ++k) {
-            const uint64_t a =
-                smem_desc_sw128(q_base + (k >> 2) * S::kQHalfBytes + (k & 3) * 32, 16, 1024);
-            const uint64_t bk =
-                smem_desc_sw128(kt + (k >> 2) * S::kHalfTileBytes + (k & 3) * 32, 16, 1024);
-            tc_mma(tmem + q * S::kTile, a, bk, id_s, k > 0);
-          }
-          tc_commit(&s_full[q]);
-          tc_commit(&k_empty[ks]);
-          if (t >= other) tc_commit(&k_empty[ks]);
-        }
-        __syncwarp();
-      }
-    } else {
-      constexpr uint32_t id_o = idesc_bf16(128, D, true);  // P from TMEM, MN-major V
-      for (int i = 0; ok && i < nt; ++i) {
-        const int t = t0 + i, vs = i % S::kVStages;
-        if (!warp_wait(&v_full[vs], (uint32_t)(i / S::kVStages) & 1u, abort_flag, wait_lim)) {
-          ok = false;
-          break;
-        }
-        if (t == ntiles - 1 && kv_end < (t + 1) * S::kTile) {
-          // slots >= kv_end get p = 0; zero their value rows so that stale bits never reach O
-          // (both O warps may write the same zeros)
-          const int z0 = kv_end - t * S::kTile, per_half = (S::kTile - z0) * 8;
-          uint8_t *vt = smem + S::kOffV + vs * S::kKVBytes;
-          for (int e = lane; e < S::kHalves * per_half; e += 32) {
-            const int hh = e / per_half, r = e % per_half;
-            *reinterpret_cast<uint4 *>(vt + hh * S::kHalfTileBytes + z0 * 128 + r * 16) =
-                make_uint4(0u, 0u, 0u, 0u);
-          }
-          fence_proxy_async_smem();
-          __syncwarp();
-        }
-        if (!warp_wait(&p_full[q], (uint32_t)i & 1u, abort_flag, wait_lim)) {
-          ok = false;
-          break;
-        }
-        if (lane == 0) {
-          tc_fence_after();
-          const uint32_t vt = smem_u32(smem + S::kOffV + vs * S::kKVBytes);
-#pragma unroll
-          for (int k = 0; k < S::kTile / 16; ++k) {
-            const uint64_t bv = smem_desc_sw128(vt + k * 2048, S::kHalfTileBytes, 1024);
-            tc_mma_tmem_a(tmem + S::kOffO + q * D, tmem + S::kOffP + q * (S::kTile / 2) + k * 8,
-                          bv, id_o, i > 0 || k > 0);
-          }
-          tc_commit(&pv_done[q]);
-          tc_commit(&v_empty[vs]);
-          if (t >= other) tc_commit(&v_empty[vs]);
-        }
-        __syncwarp();
-      }
-    }
-    if (!ok && lane == 0 && !*abort_flag) {
+  // The next item: every role reads it from the item ring and frees the entry.
+  auto give_up = [&]() {
+    if (lane == 0 && !*abort_flag) {
       record_error(v.err, HAM_DEVERR_TIMEOUT);
       *abort_flag = 1;
     }
-    // every MMA issued completes before the tensor memory is freed
-    if (lane == 0) {
-      tc_commit(mma_done);
-      thread_wait(mma_done, 0u, abort_flag, false);
+  };
+  auto next_item = [&](uint32_t k, PrefillItem &it) -> bool {
+    const uint32_t x = k % S::kItems;
+    if (!warp_wait_small(&item_full[x], (k / S::kItems) & 1u, abort_flag, kWaitLimitNs)) {
+      give_up();
+      return false;
     }
+    it = items[x];
     __syncwarp();
+    if (lane == 0) mbar_arrive(&item_empty[x]);
+    return uniform(it.valid) != 0;
+  };
+  uint32_t issued = 0, q_issued[2] = {0u, 0u};  // producers: ring entries past the last one; Q loads
+
+  if (warp >= S::kProducerWarp) {
+    if (warp < S::kMmaWarp) {
+      // ---------------------------------------------------------- producers: TMA copies
+      // One warp streams the K tiles, the other Q and the V tiles, into one ring in the order
+      // K_0 V_0 K_1 V_1 ... (the order the products read them).  A chunk at or past the item's
+      // end is not copied: its rows are never read (whole chunks) or zeroed (V, the last one).
+      const bool is_v = warp == S::kVProducerWarp;
+      const CUtensorMap *map = is_v ? &tmap_v : &tmap_k;
+      const uint64_t pol_first = policy_evict_first(), pol_last = policy_evict_last();
+      uint32_t e = is_v ? 1 : 0;  // ring entry of the next tile
+      bool ok = true;
+      PrefillItem it;
+      // The V producer hands the items out: the next one once it has issued this one's last copies
+      // (earlier would give a CTA two of the launch's last items while others have none).
+      const int nblocks = v.next_item[1];
+      const int total = Hkv * nblocks * v.splits;
+      auto fetch = [&](uint32_t k) -> bool {
+        const uint32_t x = k % S::kItems;
+        if (k >= S::kItems && !warp_wait_small(&item_empty[x], ((k / S::kItems) - 1) & 1u,
+                                               abort_flag, kWaitLimitNs)) {
+          give_up();
+          return false;
+        }
+        it = PrefillItem{};
+        for (;;) {
+          int id = 0;
+          if (lane == 0) id = atomicAdd(v.next_item, 1);
+          id = uniform(id);
+          if (id >= total || decode_item(v, id, nblocks, S::kTile, it)) break;
+        }
+        if (lane == 0) {
+          items[x] = it;
+          mbar_arrive(&item_full[x]);
+        }
+        return uniform(it.valid) != 0;
+      };
+      for (uint32_t k = 0; ok; ++k) {
+        if (is_v ? !fetch(k) : !next_item(k, it)) break;
+        const int nts = uniform(max(it.nt0, it.nt1)), kv_end = uniform(max(it.end0, it.end1));
+        // a sequence with several query blocks re-reads its K/V from L2
+        const uint64_t pol_kv = it.n > 2 * R ? pol_last : pol_first;
+        if (is_v) {  // Q (so that the K tiles do not wait for the previous item's last product)
+          const int nq = it.nt1 > 0 ? 2 : 1;
+          for (int q = 0; ok && q < nq; ++q) {
+            if (q_issued[q] > 0 &&
+                !warp_wait_small(&q_empty[q], (q_issued[q] - 1) & 1u, abort_flag, wait_lim)) {
+              give_up();
+              ok = false;
+              break;
+            }
+            ++q_issued[q];
+            if (elect_one()) {
+              mbar_arrive_tx(&q_full[q], (uint32_t)S::kQBytes);
+              tma_load_4d(smem + q * S::kQBytes, &tmap_q, 0, it.g * G, it.row0 + it.qb0 + q * R, 0,
+                          &q_full[q], pol_first);
+            }
+            __syncwarp();
+          }
+          if (!ok) break;
+        }
+        // Page-table entries of 32 chunks (4 tiles) at a time, one per lane, requested a batch
+        // ahead: lane l holds the pool row of chunk base + l (-1: at or past the item's end; -2:
+        // a page outside the pool).
+        const int nchunks = (kv_end + kChunkSlots - 1) / kChunkSlots;
+        auto lookup = [&](int base) {
+          int row = -1;
+          if (base + lane < nchunks) {
+            const int slot0 = (base + lane) * kChunkSlots;
+            const int page = v.page_table[(int64_t)it.b * v.max_pages + slot0 / v.page_slots];
+            row = page < 0 || page >= v.pool_pages
+                      ? -2
+                      : (int)(((int64_t)page * Hkv + it.g) * v.page_slots + slot0 % v.page_slots);
+          }
+          return row;
+        };
+        constexpr int kTilesPerBatch = 32 / S::kChunks;
+        const int cbase = it.t0 * S::kChunks;  // the item's first chunk
+        int row = lookup(cbase), row_next = lookup(cbase + 32);
+        for (int i = 0; i < nts; ++i, e += 2) {
+          if (i > 0 && i % kTilesPerBatch == 0) {
+            row = row_next;
+            row_next = lookup(cbase + (i / kTilesPerBatch + 1) * 32);
+          }
+          if (__any_sync(kFull, row == -2)) {  // the plan validated the table: ends the CTA
+            if (lane == 0) {
+              record_error(v.err, HAM_DEVERR_PAGE);
+              *abort_flag = 1;
+            }
+            ok = false;
+            break;
+          }
+          const uint32_t st = e % S::kStages;
+          if (e >= S::kStages && !warp_wait_small(&empty[st], ((e / S::kStages) - 1) & 1u,
+                                                 abort_flag, wait_lim)) {
+            give_up();
+            ok = false;
+            break;
+          }
+          const int nck = min(S::kChunks, nchunks - cbase - i * S::kChunks);
+          const int at = (i % kTilesPerBatch) * S::kChunks;
+          if (elect_one()) mbar_arrive_tx(&full[st], (uint32_t)(nck * kChunkSlots * D * 2));
+          uint8_t *dst = smem + S::kOffRing + st * S::kKVBytes;
+#pragma unroll 1
+          for (int c = 0; c < nck; ++c) {
+            const int r = __shfl_sync(kFull, row, at + c);
+            if (elect_one()) tma_load_4d(dst + c * S::kChunkBytes, map, 0, 0, 0, r >> 3, &full[st], pol_kv);
+          }
+        }
+      }
+      issued = e;
+    } else {
+      // ---------------------------------------------------------- MMA issue (one thread a Q tile)
+      // The first S of an item (two where S goes by blocks), then block by block O += P V once the
+      // softmax group has written P, and the S whose columns are free then.  What holds an item's
+      // end takes only the 16-slot chunks it reaches (N of S, K of P V).  Both warps release every
+      // K and V stage: by a commit after the products that read it, or by an arrival where their Q
+      // tile has none, so that neither falls a ring's turn behind.  Everything the products'
+      // operands depend on is kept uniform over the warp: with per-thread values an issue took
+      // about 100 cycles, against the 32 to 64 that the product itself takes.
+      constexpr uint32_t id_o = idesc_bf16(128, D, true);  // P from TMEM, MN-major V
+      const int q = warp - S::kMmaWarp;
+      const uint32_t ring = smem_u32(smem + S::kOffRing);
+      const uint64_t q_desc = smem_desc_sw128(smem_u32(smem) + q * S::kQBytes, 16, 1024);
+      const uint32_t d_s = tmem + q * S::kTile, d_o = tmem + S::kOffO + q * D;
+      uint32_t e = 0, pc = 0, qc = 0;  // ring entry of the item's first K tile; parities of P; Q loads
+      bool ok = true;
+      PrefillItem it;
+      for (uint32_t k = 0; ok && next_item(k, it); ++k) {
+        const int nt = uniform(q ? it.nt1 : it.nt0), nts = uniform(max(it.nt0, it.nt1));
+        const int base = uniform(it.t0) * S::kTile, end = uniform(q ? it.end1 : it.end0) - base;
+        const int kv_end = uniform(max(it.end0, it.end1)) - base;  // (from the item's first slot)
+        // blocks of this Q tile (a tile without rows has no end)
+        const int nb = nt == 0 ? 0 : min(2 * nt, (end + S::kBlock - 1) / S::kBlock);
+        const uint32_t e0 = e;
+        e += 2 * nts;
+        auto chunks = [&](int from, int most) {  // 16-slot chunks that this Q tile reaches
+          return min(most, (end - from + kChunkSlots - 1) / kChunkSlots);
+        };
+        auto wait_entry = [&](uint32_t x) {
+          return warp_wait_small(&full[x % S::kStages], (x / S::kStages) & 1u, abort_flag, wait_lim);
+        };
+        // S of tile t / 2 or of block t, and the release of K and Q after their last.
+        auto issue_s = [&](int t) {
+          const uint32_t st = (e0 + 2 * (t >> 1)) % S::kStages, buf = S::kTileS ? 0 : t & 1;
+          const uint64_t b0 = smem_desc_sw128(
+              ring + st * S::kKVBytes + buf * (S::kBlock / 8) * S::kGroupBytes, 16, S::kGroupBytes);
+          const uint32_t id_s = idesc_bf16(
+              128, kChunkSlots * chunks(t * S::kBlock, S::kSSlots / kChunkSlots), false);  // K-major
+#pragma unroll
+          for (int kk = 0; kk < D / 16; ++kk)
+            tc_mma(d_s + buf * S::kBlock,
+                   q_desc + (uint64_t)(((kk >> 2) * S::kQHalfBytes + (kk & 3) * 32) >> 4),
+                   b0 + (uint64_t)(((kk >> 2) * 1024 + (kk & 3) * 32) >> 4), id_s, kk > 0);
+          tc_commit(&s_full[2 * q + buf]);
+          const bool last = t + (S::kTileS ? 2 : 1) >= nb;
+          if (S::kTileS || buf == 1 || last) tc_commit(&empty[st]);
+          if (last) tc_commit(&q_empty[q]);
+        };
+        if (nb > 0) {
+          ok = warp_wait_small(&q_full[q], qc & 1u, abort_flag, wait_lim);
+          if (!ok) break;
+          ok = wait_entry(e0);
+          if (!ok) break;
+          ++qc;
+          tc_fence_after();
+          if (elect_one()) issue_s(0);
+          __syncwarp();
+          if (!S::kTileS && nb > 1 && elect_one()) issue_s(1);
+          __syncwarp();
+        }
+        for (int t = 0; t < nb; ++t) {
+          const uint32_t buf = t & 1, ev = e0 + 2 * (t >> 1) + 1, sv = ev % S::kStages;  // V's entry
+          if (buf == 0) {  // a new tile: its values, and the keys of the next one
+            ok = wait_entry(ev);
+            if (!ok) break;
+            if ((t >> 1) + 1 < nt) {
+              ok = wait_entry(ev + 1);
+              if (!ok) break;
+            }
+            const int z0 = kv_end - t * S::kBlock;  // rows of the tile >= z0 are past the last slot
+            if (z0 < S::kTile && (z0 & (kChunkSlots - 1))) {
+              // slots past the end get p = 0; zero their value rows (to the end of the last chunk
+              // the products read) so that stale bits never reach O (both warps may do it)
+              uint8_t *vt = smem + S::kOffRing + sv * S::kKVBytes;
+              const int pieces = (kChunkSlots - (z0 & (kChunkSlots - 1))) * S::kHalves * 8;
+              for (int x = lane; x < pieces; x += 32) {  // 16-byte pieces of rows z0 ..
+                const int row = z0 + x / (S::kHalves * 8), y = x % (S::kHalves * 8);
+                *reinterpret_cast<uint4 *>(vt + (row >> 3) * S::kGroupBytes + (y >> 3) * 1024 +
+                                           (row & 7) * 128 + (y & 7) * 16) = make_uint4(0u, 0u, 0u, 0u);
+              }
+              fence_proxy_async_smem();
+              __syncwarp();
+            }
+          }
+          ok = warp_wait_small(&p_full[2 * q + buf], (pc >> buf) & 1u, abort_flag, wait_lim);
+          if (!ok) break;
+          pc ^= 1u << buf;
+          tc_fence_after();
+          const int nc = chunks(t * S::kBlock, S::kBlockChunks);
+          const uint32_t a0 = d_s + buf * S::kBlock;
+          const uint64_t v0 = smem_desc_sw128(  // MN-major: halves 1024 bytes apart
+              ring + sv * S::kKVBytes + buf * (S::kBlockChunks * S::kChunkBytes), 1024, S::kGroupBytes);
+          if (elect_one()) {
+#pragma unroll
+            for (int c = 0; c < S::kBlockChunks; ++c)
+              if (c < nc)
+                tc_mma_tmem_a(d_o, a0 + c * 8, v0 + (uint64_t)(c * S::kChunkBytes >> 4), id_o,
+                              t > 0 || c > 0);
+            tc_commit(&pv_done[q]);
+            if (t + 1 == nb) tc_commit(&o_full[q]);
+            if (S::kTileS) {
+              if (buf == 1 && t + 1 < nb) issue_s(t + 1);
+            } else if (t + 2 < nb) {
+              issue_s(t + 2);
+            }
+            if (buf == 1 || t + 1 == nb) tc_commit(&empty[sv]);
+          }
+          __syncwarp();
+        }
+        for (uint32_t x = e0 + 2 * nt; ok && x != e; ++x) {  // tiles it does not reach
+          ok = wait_entry(x);
+          if (ok && lane == 0) mbar_arrive(&empty[x % S::kStages]);
+        }
+      }
+      if (!ok) give_up();
+      // every MMA issued completes before the tensor memory is freed
+      if (elect_one()) {
+        tc_commit(mma_done);
+        thread_wait(mma_done, 0u, abort_flag, false);
+      }
+      __syncwarp();
+    }
   } else {
     // ------------------------------------------------------------ softmax groups
     // Thread = TMEM lane = row m of Q tile q.  Each row's scores arrive whole in its own thread,
     // so the row maximum and sum need no shuffles.
     const int q = warp >> 2, m = tid & 127;
     const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
-    const uint32_t t_s = tmem + lane_base + q * S::kTile;
-    const uint32_t t_p = tmem + lane_base + S::kOffP + q * (S::kTile / 2);
+    const uint32_t t_s = tmem + lane_base + q * S::kTile;  // the two blocks of S_q, then P_q
     const uint32_t t_o = tmem + lane_base + S::kOffO + q * D;
-    const int j = qb0 + q * R + m / G;          // the row's index in the sequence's chunk
-    const int lim = L + min(j, n - 1);          // last slot it attends (rows past n: not stored)
-    const int lim_min = L + qb0 + q * R;        // smallest limit of the tile's stored rows
     const float sl2 = (float)(1.4426950408889634 / sqrt((double)D));  // 1/sqrt(d), log2(e)
-    float m_run = -INFINITY, l_run = 0.f;
+    uint32_t sp = 0, np = 0, oc = 0, turns = 0;  // phase parities of s_full; blocks, items, turns so far
     bool ok = true;
-    for (int i = 0; i < ntq[q]; ++i) {
-      const int t = t0 + i;
-      if (!warp_wait(&s_full[q], (uint32_t)i & 1u, abort_flag, wait_lim)) {
+    for (uint32_t k = 0;; ++k) {
+      int tbase, tend, lim, lim_min;  // first slot of the block, of the item's end; row limits
+      int take_lo, take_hi, give_hi;  // tiles (first slots) that take and give the turn
+      int64_t orow = -1;              // the row's place in out (or in the split's partials)
+      bool whole;
+      {
+        PrefillItem it;
+        if (!next_item(k, it)) break;
+        const int nt = q ? it.nt1 : it.nt0;
+        if (nt == 0) continue;
+        const int j = it.qb0 + q * R + m / G;  // the row's index in the sequence's chunk
+        lim = it.L + min(j, it.n - 1);         // last slot it attends (rows past n: not stored)
+        lim_min = it.L + it.qb0 + q * R;       // smallest limit of the tile's stored rows
+        tbase = it.t0 * S::kTile;
+        tend = min(tbase + nt * S::kTile, q ? it.end1 : it.end0);
+        whole = it.zs == 1;
+        // Turns, in the tiles that both Q tiles read: Q tile 1's softmax of a tile follows Q tile 0's,
+        // which follows Q tile 1's of the tile before.
+        const int both = it.nt1 > 0 ? tbase + it.nt0 * S::kTile : tbase;  // end of those tiles
+        take_lo = tbase + (q == 0 ? S::kTile : 0);
+        take_hi = both;
+        give_hi = both - (q == 0 ? 0 : S::kTile);
+        if (j < it.n)
+          orow = ((whole ? 0 : (int64_t)it.z * v.rows) + it.row0 + j) * Hq + it.g * G + m % G;
+      }
+      float m_run = -INFINITY, l_run = 0.f;
+      for (uint32_t buf = 0; tbase < tend; tbase += S::kBlock, buf ^= 1u, ++np) {
+        if (!S::kTileS || buf == 0) {  // new scores
+          if (!warp_wait_small(&s_full[2 * q + buf], (sp >> buf) & 1u, abort_flag, wait_lim)) {
+            ok = false;
+            break;
+          }
+          sp ^= 1u << buf;
+          if (S::kTileS && tbase >= take_lo && tbase < take_hi) {
+            if (!warp_wait_small(&turn[q], turns & 1u, abort_flag, wait_lim)) {
+              ok = false;
+              break;
+            }
+            ++turns;
+          }
+          tc_fence_after();
+        }
+        const uint32_t t_b = t_s + buf * S::kBlock;
+        uint32_t r[2][32];
+        tmem_ld32(t_b, r[0]);
+        tmem_ld32(t_b + 32, r[1]);
+        tmem_wait_ld();
+        if (tbase + S::kBlock - 1 > lim_min) mask_scores(r, lim - tbase);
+        // Running maximum in the exp2 domain, raised lazily: only when a score passes it by more
+        // than kRescaleSlack (p then stays below 2^kRescaleSlack), so O is rarely rescaled.  The
+        // item's first block always raises it (its first slot is attended by every row).
+        const float mx = max_score(r) * sl2;
+        const bool raise = mx > m_run + kRescaleSlack;
+        if (__any_sync(kFull, raise)) {
+          const float alpha = raise ? ex2(m_run - mx) : 1.f;
+          if (__any_sync(kFull, raise && m_run != -INFINITY)) {  // (the first block overwrites O)
+            // once O holds the previous block too (the phase before this block's)
+            if (!warp_wait_small(&pv_done[q], (np - 1) & 1u, abort_flag, wait_lim)) {
+              ok = false;
+              break;
+            }
+            tc_fence_after();
+#pragma unroll 1
+            for (int c0 = 0; c0 < D; c0 += 32) {
+              uint32_t o[32];
+              tmem_ld32(t_o + c0, o);
+              tmem_wait_ld();
+#pragma unroll
+              for (int x = 0; x < 32; ++x) o[x] = __float_as_uint(__uint_as_float(o[x]) * alpha);
+              tmem_st32(t_o + c0, o);
+            }
+          }
+          if (raise) m_run = mx;
+          l_run *= alpha;
+        }
+        // P in two parts, the first stored while the second is formed (in one part: 8% slower)
+        float rs0 = 0.f, rs1 = 0.f, rs2 = 0.f, rs3 = 0.f;
+#pragma unroll
+        for (int x = 0; x < 2; ++x) {
+          uint32_t pk[16];
+#pragma unroll
+          for (int c = 0; c < 32; c += 4) {
+            const float p0 = ex2(fmaf(__uint_as_float(r[x][c]), sl2, -m_run));
+            const float p1 = ex2(fmaf(__uint_as_float(r[x][c + 1]), sl2, -m_run));
+            const float p2 = ex2(fmaf(__uint_as_float(r[x][c + 2]), sl2, -m_run));
+            const float p3 = ex2(fmaf(__uint_as_float(r[x][c + 3]), sl2, -m_run));
+            rs0 += p0;
+            rs1 += p1;
+            rs2 += p2;
+            rs3 += p3;
+            pk[c / 2] = pack_bf16x2(p0, p1);
+            pk[c / 2 + 1] = pack_bf16x2(p2, p3);
+          }
+          if (x == 1 && S::kTileS && (buf == 1 || tbase + S::kBlock >= tend) &&
+              tbase - (int)buf * S::kBlock < give_hi && lane == 0)
+            mbar_arrive(&turn[q ^ 1]);
+          tmem_st16(t_b + 16 * x, pk);  // 32 probabilities as 16 bf16 pairs
+        }
+        l_run += (rs0 + rs1) + (rs2 + rs3);
+        tmem_wait_st();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&p_full[2 * q + buf]);
+      }
+      if (!ok || !warp_wait_small(&o_full[q], oc & 1u, abort_flag, wait_lim)) {
         ok = false;
         break;
       }
+      ++oc;
       tc_fence_after();
-      float s[S::kTile];
-#pragma unroll
-      for (int c0 = 0; c0 < S::kTile; c0 += 32) {
-        uint32_t r[32];
-        tmem_ld32(t_s + c0, r);
-#pragma unroll
-        for (int c = 0; c < 32; ++c) s[c0 + c] = __uint_as_float(r[c]);
-      }
-      tmem_wait_ld();
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&s_free[q]);  // the next scores may overwrite S_q
-      const int tbase = t * S::kTile;
-      if (tbase + S::kTile - 1 > lim_min) {  // the causal edge (and the chunk's end) in this tile
-#pragma unroll
-        for (int c = 0; c < S::kTile; ++c)
-          if (tbase + c > lim) s[c] = -INFINITY;
-      }
-      float mx;
-      {  // tree maximum
-        float r[16];
-#pragma unroll
-        for (int c = 0; c < 16; ++c)
-          r[c] = fmaxf(fmaxf(s[c], s[c + 16]), fmaxf(s[c + 32], s[c + 48]));
-#pragma unroll
-        for (int w = 8; w > 0; w >>= 1)
-#pragma unroll
-          for (int c = 0; c < w; ++c) r[c] = fmaxf(r[c], r[c + w]);
-        mx = r[0] * sl2;
-      }
-      // Running maximum in the exp2 domain, raised lazily: only when a score passes it by more
-      // than kRescaleSlack (p then stays below 2^kRescaleSlack), so O is rarely rescaled.  The
-      // split's first tile always raises it (its first slot is attended by every row).
-      float alpha = 1.f;
-      if (mx > m_run + kRescaleSlack) {
-        alpha = ex2(m_run - mx);
-        m_run = mx;
-      }
-      uint32_t pk[S::kTile / 2];
-      float rs0 = 0.f, rs1 = 0.f, rs2 = 0.f, rs3 = 0.f;
-#pragma unroll
-      for (int c = 0; c < S::kTile; c += 4) {
-        const float p0 = ex2(fmaf(s[c], sl2, -m_run));
-        const float p1 = ex2(fmaf(s[c + 1], sl2, -m_run));
-        const float p2 = ex2(fmaf(s[c + 2], sl2, -m_run));
-        const float p3 = ex2(fmaf(s[c + 3], sl2, -m_run));
-        rs0 += p0;
-        rs1 += p1;
-        rs2 += p2;
-        rs3 += p3;
-        pk[c / 2] = pack_bf16x2(p0, p1);
-        pk[c / 2 + 1] = pack_bf16x2(p2, p3);
-      }
-      l_run = l_run * alpha + ((rs0 + rs1) + (rs2 + rs3));
-      // O_q and P_q are free once the previous product has completed
-      if (i > 0) {
-        if (!warp_wait(&pv_done[q], (uint32_t)(i - 1) & 1u, abort_flag, wait_lim)) {
-          ok = false;
-          break;
+      if (whole) {  // normalised output
+        const float inv = l_run > 0.f ? 1.f / l_run : 0.f;
+        OutT *dst = static_cast<OutT *>(v.out) + orow * D;
+#pragma unroll 1
+        for (int c0 = 0; c0 < D; c0 += 32) {
+          uint32_t o[32];
+          tmem_ld32(t_o + c0, o);
+          tmem_wait_ld();
+          if (orow >= 0) store_row32<OutT>(dst + c0, o, inv);
         }
-        tc_fence_after();
-        if (__any_sync(kFull, alpha != 1.f)) {  // rescale O (some row of the warp raised its max)
-#pragma unroll
-          for (int c0 = 0; c0 < D; c0 += 32) {
-            uint32_t o[32];
-            tmem_ld32(t_o + c0, o);
-            tmem_wait_ld();
-#pragma unroll
-            for (int e = 0; e < 32; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha);
-            tmem_st32(t_o + c0, o);
-          }
+      } else {  // this split's partial: O in units of 2^m_run, the running max and sum
+        float *dst = v.part_o + orow * D;
+#pragma unroll 1
+        for (int c0 = 0; c0 < D; c0 += 32) {
+          uint32_t o[32];
+          tmem_ld32(t_o + c0, o);
+          tmem_wait_ld();
+          if (orow >= 0) store_row32<float>(dst + c0, o, 1.f);
         }
-      }
-      tmem_st32(t_p, pk);  // P_q: the tile's 64 probabilities as 32 bf16 pairs
-      tmem_wait_st();
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&p_full[q]);
-    }
-    if (ok && ntq[q] > 0) {
-      if (!warp_wait(&pv_done[q], (uint32_t)(ntq[q] - 1) & 1u, abort_flag, wait_lim)) {
-        ok = false;
-      } else {
-        tc_fence_after();
-        const int64_t rh = (row0 + j) * Hq + g * G + m % G;  // (row, head) of the call
-        if (zs == 1) {  // the whole row: normalised output
-          const float inv = l_run > 0.f ? 1.f / l_run : 0.f;
-          OutT *orow = static_cast<OutT *>(v.out) + rh * (int64_t)D;
-#pragma unroll
-          for (int c0 = 0; c0 < D; c0 += 32) {
-            uint32_t o[32];
-            tmem_ld32(t_o + c0, o);
-            tmem_wait_ld();
-            if (j < n) store_row32<OutT>(orow + c0, o, inv);
-          }
-        } else {  // this split's partial: O in units of 2^m_run, the running max and sum
-          const int64_t pr = (int64_t)z * v.rows * Hq + rh;
-          float *prow = v.part_o + pr * D;
-#pragma unroll
-          for (int c0 = 0; c0 < D; c0 += 32) {
-            uint32_t o[32];
-            tmem_ld32(t_o + c0, o);
-            tmem_wait_ld();
-            if (j < n) store_row32<float>(prow + c0, o, 1.f);
-          }
-          if (j < n) v.part_ml[pr] = make_float2(m_run, l_run);
-        }
+        if (orow >= 0) v.part_ml[orow] = make_float2(m_run, l_run);
       }
     }
-    if (!ok && lane == 0 && !*abort_flag) {
-      record_error(v.err, HAM_DEVERR_TIMEOUT);
-      *abort_flag = 1;
-    }
+    if (!ok) give_up();
   }
   // all tensor-memory reads and MMAs are done: free the columns
+  volatile uint32_t *issued_s = reinterpret_cast<volatile uint32_t *>(items);  // K, V, Q tiles
   tc_fence_before();
   __syncthreads();
-  if (warp == S::kSWarp0) {
+  if (lane == 0 && warp == S::kProducerWarp) issued_s[0] = issued;
+  if (lane == 0 && warp == S::kVProducerWarp) {
+    issued_s[1] = issued;
+    issued_s[2] = q_issued[0];
+    issued_s[3] = q_issued[1];
+  }
+  if (warp == S::kMmaWarp) {
     tc_fence_after();
     tmem_dealloc<S::kTmemCols>(tmem);
+  }
+  __syncthreads();
+  if (tid == 0 && *abort_flag) {
+    // after an abort, every copy this CTA issued lands before the CTA can exit (without one, the
+    // MMA warp waited for every copy): the entries whose ring stage was not filled again
+    for (uint32_t w = 0; w < 2; ++w)
+      for (uint32_t x = w; x < issued_s[w]; x += 2) {
+        const uint32_t y = x + S::kStages;  // the entry that would reuse the stage
+        if (y >= issued_s[y & 1]) thread_wait(&full[x % S::kStages], (x / S::kStages) & 1u, abort_flag, false);
+      }
+    for (int q = 0; q < 2; ++q)
+      if (issued_s[2 + q] > 0) thread_wait(&q_full[q], (issued_s[2 + q] - 1) & 1u, abort_flag, false);
   }
 }
 
@@ -885,12 +1059,11 @@ cudaError_t launch_attn(const CUtensorMap &tq, const CUtensorMap &tk, const CUte
   cudaError_t e = cudaFuncSetAttribute(prefill_attn_kernel<D, OutT>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, S::kSmem);
   if (e != cudaSuccess) return e;
-  const int QB = prefill_query_rows(v.n_q_heads / v.n_kv_heads);
-  const int Z = v.splits < 1 ? 1 : v.splits;
-  const dim3 grid((unsigned)v.n_kv_heads, (unsigned)(v.rows / QB + v.batch), (unsigned)Z);
+  const int64_t items = (int64_t)v.n_kv_heads * v.blocks * v.splits;
+  const unsigned grid = (unsigned)(items < v.sms ? items : v.sms);  // persistent: one CTA an SM
   prefill_attn_kernel<D, OutT><<<grid, S::kThreads, S::kSmem, stream>>>(tq, tk, tv, v);
   e = cudaGetLastError();
-  if (e != cudaSuccess || Z == 1) return e;
+  if (e != cudaSuccess || v.splits == 1) return e;
   const int64_t pairs = (int64_t)v.rows * v.n_q_heads;
   prefill_merge_kernel<OutT><<<(unsigned)((pairs + kMergeWarps - 1) / kMergeWarps),
                                kMergeWarps * 32, 0, stream>>>(v);

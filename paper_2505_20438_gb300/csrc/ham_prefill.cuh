@@ -21,8 +21,8 @@ struct PrefillView {
   const uint16_t *k_new, *v_new;
   const int32_t *offsets, *pos, *ntok;  // pos, ntok nullable
   void *out;                   // [rows][n_q_heads][head_dim], bf16 or f32
-  int4 *seq_info;              // scratch [batch]: (first new slot or -1, rows, query-block
-                               // start, 1 when the call's offsets are valid, else 0)
+  int4 *seq_info;              // scratch [batch]: (first new slot or -1, rows, unused, 1 when the
+                               // call's offsets are valid, else 0)
   int2 *row_info;              // scratch [rows]: (position, pool row page * page_slots + row
                                // in page, or -1 when the row is not stored) of each new row
   int32_t *err;
@@ -37,14 +37,30 @@ struct PrefillView {
   float *part_o;
   float2 *part_ml;
   int32_t splits;
+  // The attention's work items, KV heads x query blocks x splits: query blocks of the call at most,
+  // their order [blocks] (sequence, block of its chunk), the counter the items are handed out from
+  // and, after it, the number of query blocks (scratch, all written by the plan); SMs of the device.
+  int32_t blocks;
+  int2 *order;
+  int32_t *next_item;
+  int32_t sms;
 };
-// Slots a prefill split covers at least (whole 64-slot tiles of the cached part), and the most
-// splits a launch uses.
-constexpr int kPrefillSplitMinTiles = 8, kPrefillMaxSplits = 32;
+// One work item of the attention kernel: two Q tiles of a KV head over a range of K/V tiles.
+struct alignas(16) PrefillItem {
+  int32_t valid;               // 0: no more items
+  int32_t b, g;                // sequence, KV head
+  int32_t L, n, qb0, row0;     // cached slots, the chunk's rows, the item's first row; call row 0
+  int32_t z, zs;               // split z of zs
+  int32_t t0, nt0, nt1;        // first K/V tile; tiles Q tile 0 / 1 reads (nt1 = 0 or >= nt0)
+  int32_t end0, end1;          // first slot no row of Q tile 0 / 1 attends (end1 = 0: no rows)
+};
+// Cached slots a prefill split covers at least, the most splits and the most query blocks of a
+// launch.
+constexpr int kPrefillSplitMinSlots = 512, kPrefillMaxSplits = 32, kPrefillMaxBlocks = 65535;
 // Splits of a sequence holding L cached slots, at most Z: each takes at least
-// kPrefillSplitMinTiles tiles of the cached part, the last one also the chunk's own slots.
+// kPrefillSplitMinSlots of them, the last one also the chunk's own slots.
 __host__ __device__ inline int prefill_splits(int L, int Z) {
-  const int by_len = (L / 64) / kPrefillSplitMinTiles;
+  const int by_len = L / kPrefillSplitMinSlots;
   return by_len < 1 ? 1 : (by_len < Z ? by_len : Z);
 }
 // Scratch floats the split partials may use: SMs x 256 (row, head) pairs x head_dim (a launch
@@ -55,7 +71,12 @@ inline size_t prefill_part_floats(int sms, int head_dim) {
 cudaError_t launch_prefill(const CUtensorMap &tk, const CUtensorMap &tv, const PrefillView &v,
                            int out_dtype, cudaStream_t stream);
 bool prefill_supported(int head_dim, int group);
-// Query rows of one sequence that one prefill attention CTA covers (128 / group).
+// Query rows of one sequence that one prefill attention item covers (two tiles of 128 / group).
 int prefill_query_rows(int group);
+// Query blocks of a call of `rows` rows over `batch` sequences, at most: the sum over the sequences
+// of ceil(rows of the sequence / qb_rows).
+inline int64_t prefill_blocks(int64_t rows, int64_t batch, int qb_rows) {
+  return (rows + batch * (qb_rows - 1)) / qb_rows;
+}
 
 }  // namespace ham

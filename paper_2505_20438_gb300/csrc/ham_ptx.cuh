@@ -438,6 +438,33 @@ __device__ bool warp_wait(uint64_t *bar, uint32_t parity, volatile int *abort_fl
   }
 }
 
+// The same wait in few instructions (kernels whose hot loops wait at many places: their code has
+// to stay in the instruction cache), every lane keeping the time.
+__device__ __forceinline__ bool warp_wait_small(uint64_t *bar, uint32_t parity,
+                                                volatile int *abort_flag, uint64_t limit_ns) {
+  const bool brief = limit_ns < kWaitLimitNs;  // shortened: poll without suspending
+  uint64_t t0 = 0;
+#pragma unroll 1
+  for (uint32_t n = 0;; ++n) {
+    if (__all_sync(kFull, brief ? mbar_poll(bar, parity) : mbar_test(bar, parity)))
+      return true;
+    if (n == 0) t0 = global_timer_ns();
+    else if ((brief || (n & 15u) == 0) &&
+             __any_sync(kFull, *abort_flag != 0 || global_timer_ns() - t0 > limit_ns))
+      return false;
+  }
+}
+// True in one thread of the (converged) warp.  Code under it issues tcgen05 and TMA instructions
+// with their operands in uniform registers, which a lane-number test does not allow.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n .reg .pred P;\n elect.sync _|P, 0xffffffff;\n selp.b32 %0, 1, 0, P;\n}"
+               : "=r"(p));
+  return p != 0;
+}
+// The value of lane 0, known to be the same in the whole warp.
+__device__ __forceinline__ int uniform(int x) { return __shfl_sync(kFull, x, 0); }
+
 // Byte offset of the 16-byte piece `c` (elements 8c .. 8c+7) of row `row` in a tile written by a
 // TMA copy with the 128-byte swizzle: rows are split into 128-byte lines (line = row *
 // lines_per_row + c / 8) and the piece index inside a line is XORed with line % 8.  The tile

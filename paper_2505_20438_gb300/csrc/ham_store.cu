@@ -166,6 +166,7 @@ void note_launch(const ham_kv *kv, int32_t layer, void *stream, bool writes) {
 // handle keeps no pointer to.
 struct MetaLayout {
   size_t pos, ntok, pt, ns, nt, inv_freq, err, acc, ml, sr, stash, arrive, pf_seq, pf_pos;
+  size_t pf_next, pf_order;  // ham_prefill: item counter and block count; order of the query blocks
   size_t pf_part, pf_ml;  // ham_prefill's split partials (bf16 caches; empty for FP8)
   size_t front_stage;     // ham_qkv_append on FP8 caches: the new rows as bf16 (else empty)
   size_t front_enc;       // ... and the per-head arrival counters of its encoding
@@ -199,6 +200,12 @@ MetaLayout meta_layout(const ham_config &cfg, int32_t max_ctas, int64_t max_page
   m.arrive = carve(sizeof(int32_t));
   m.pf_seq = carve((size_t)cfg.batch * sizeof(int4));
   m.pf_pos = carve((size_t)cfg.batch * cfg.max_slots_per_seq * sizeof(int2));
+  m.pf_next = carve(2 * sizeof(int32_t));
+  m.pf_order = carve((size_t)std::min<int64_t>(
+                         ham::kPrefillMaxBlocks,
+                         ham::prefill_blocks((int64_t)cfg.batch * cfg.max_slots_per_seq, cfg.batch,
+                                             ham::prefill_query_rows(group))) *
+                     sizeof(int2));
   {  // (max_ctas is 8 x the SMs)
     const bool fp8 = cfg.kv_dtype == HAM_KV_E4M3;
     const size_t floats = fp8 ? 0 : ham::prefill_part_floats(max_ctas / 8, cfg.head_dim);
@@ -358,13 +365,27 @@ int make_rows_tensor_map(CUtensorMap *map, const void *base, int64_t rows, int h
                          int head_dim, int box_heads, int box_rows) {
   EncodeTiled encode = tensor_map_encoder();
   if (!encode) return -1;
-  const cuuint64_t dims[4] = {64, (cuuint64_t)(head_dim / 64), (cuuint64_t)heads,
-                              (cuuint64_t)rows};
-  const cuuint64_t strides[3] = {128, (cuuint64_t)head_dim * 2,
-                                 (cuuint64_t)heads * head_dim * 2};  // bytes, dims 1..3
-  const cuuint32_t box[4] = {64, 1, (cuuint32_t)box_heads, (cuuint32_t)box_rows};
+  const cuuint64_t dims[4] = {64, (cuuint64_t)heads, (cuuint64_t)rows, (cuuint64_t)(head_dim / 64)};
+  const cuuint64_t strides[3] = {(cuuint64_t)head_dim * 2, (cuuint64_t)heads * head_dim * 2,
+                                 128};  // bytes, dims 1..3
+  const cuuint32_t box[4] = {64, (cuuint32_t)box_heads, (cuuint32_t)box_rows,
+                             (cuuint32_t)(head_dim / 64)};
   const cuuint32_t estride[4] = {1, 1, 1, 1};
   return (int)encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void *>(base), dims,
+                     strides, box, estride, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                     CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+}
+
+int make_pool_group_tensor_map(CUtensorMap *map, const void *pool, int64_t rows, int head_dim) {
+  EncodeTiled encode = tensor_map_encoder();
+  if (!encode) return -1;
+  const int halves = head_dim / 64;
+  const cuuint64_t dims[4] = {64, 8, (cuuint64_t)halves, (cuuint64_t)(rows / 8)};
+  const cuuint64_t strides[3] = {(cuuint64_t)head_dim * 2, 128, (cuuint64_t)head_dim * 16};
+  const cuuint32_t box[4] = {64, 8, (cuuint32_t)halves, (cuuint32_t)(kChunkSlots / 8)};
+  const cuuint32_t estride[4] = {1, 1, 1, 1};
+  return (int)encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void *>(pool), dims,
                      strides, box, estride, CU_TENSOR_MAP_INTERLEAVE_NONE,
                      CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                      CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
@@ -423,14 +444,12 @@ int make_fp8_v_tensor_map(CUtensorMap *map, const void *v_codes, int64_t rows_d,
                      CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
 }
 
-int make_pool_tensor_map(CUtensorMap *map, const void *pool, int64_t rows, int head_dim,
-                         bool half_box) {
+int make_pool_tensor_map(CUtensorMap *map, const void *pool, int64_t rows, int head_dim) {
   EncodeTiled encode = tensor_map_encoder();
   if (!encode) return -1;
   const cuuint64_t dims[3] = {64, (cuuint64_t)(head_dim / 64), (cuuint64_t)rows};
   const cuuint64_t strides[2] = {128, (cuuint64_t)head_dim * 2};  // bytes, dims 1 and 2
-  const cuuint32_t box[3] = {64, half_box ? 1u : (cuuint32_t)(head_dim / 64),
-                             (cuuint32_t)kChunkSlots};
+  const cuuint32_t box[3] = {64, (cuuint32_t)(head_dim / 64), (cuuint32_t)kChunkSlots};
   const cuuint32_t estride[3] = {1, 1, 1};
   return (int)encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(pool), dims,
                      strides, box, estride, CU_TENSOR_MAP_INTERLEAVE_NONE,
@@ -571,6 +590,8 @@ int ham_kv_alloc(const ham_config *cfg_in, ham_kv **out) {
   kv->arrive = reinterpret_cast<int32_t *>(kv->meta + lay.arrive);
   kv->prefill_seq = reinterpret_cast<int4 *>(kv->meta + lay.pf_seq);
   kv->prefill_rows = reinterpret_cast<int2 *>(kv->meta + lay.pf_pos);
+  kv->prefill_next = reinterpret_cast<int32_t *>(kv->meta + lay.pf_next);
+  kv->prefill_order = reinterpret_cast<int2 *>(kv->meta + lay.pf_order);
   if (!kv->fp8) {
     kv->prefill_part = reinterpret_cast<float *>(kv->meta + lay.pf_part);
     kv->prefill_part_ml = reinterpret_cast<float2 *>(kv->meta + lay.pf_ml);
@@ -632,16 +653,16 @@ int ham_kv_alloc(const ham_config *cfg_in, ham_kv **out) {
     return rc;
   }
   kv->tmaps.resize((size_t)cfg.layers * 2);
-  kv->tmaps_half.resize((size_t)cfg.layers * 2);
+  kv->tmaps_group.resize((size_t)cfg.layers * 2);
   const int64_t rows = cfg.pool_pages * cfg.n_kv_heads * (int64_t)cfg.page_slots;
   for (int layer = 0; layer < cfg.layers; ++layer) {
-    if (kv->fp8) {  // the code blocks; the half-box maps (prefill) stay unused
+    if (kv->fp8) {  // the code blocks; the prefill's maps stay unused
       const ham::Fp8Layer f = ham::fp8_layer(kv->pool, rows, layer);
       int r = ham::make_fp8_k_tensor_map(&kv->tmaps[(size_t)layer * 2], f.k, rows);
       if (r == 0)
         r = ham::make_fp8_v_tensor_map(&kv->tmaps[(size_t)layer * 2 + 1], f.v,
                                        rows / cfg.page_slots * ham::kFp8HeadDim, cfg.page_slots);
-      memset(&kv->tmaps_half[(size_t)layer * 2], 0, 2 * sizeof(CUtensorMap));
+      memset(&kv->tmaps_group[(size_t)layer * 2], 0, 2 * sizeof(CUtensorMap));
       if (r != 0) {
         ham_kv_free(kv);
         return fail(HAM_ECUDA, "cuTensorMapEncodeTiled failed (CUresult %d)", r);
@@ -650,10 +671,10 @@ int ham_kv_alloc(const ham_config *cfg_in, ham_kv **out) {
     }
     for (int which = 0; which < 2; ++which) {
       int r = ham::make_pool_tensor_map(&kv->tmaps[(size_t)layer * 2 + which],
-                                        layer_pool(kv, layer, which), rows, cfg.head_dim, false);
+                                        layer_pool(kv, layer, which), rows, cfg.head_dim);
       if (r == 0)
-        r = ham::make_pool_tensor_map(&kv->tmaps_half[(size_t)layer * 2 + which],
-                                      layer_pool(kv, layer, which), rows, cfg.head_dim, true);
+        r = ham::make_pool_group_tensor_map(&kv->tmaps_group[(size_t)layer * 2 + which],
+                                            layer_pool(kv, layer, which), rows, cfg.head_dim);
       if (r != 0) {
         ham_kv_free(kv);
         return fail(HAM_ECUDA, "cuTensorMapEncodeTiled failed (CUresult %d)", r);
@@ -1046,10 +1067,10 @@ int ham_prefill(ham_kv *kv, int32_t layer, void *q_inout, const void *k_new, con
       overlaps(out, out_bytes, kv->pool, pool_bytes) || overlaps(k_new, kv_bytes, kv->pool, pool_bytes) ||
       overlaps(v_new, kv_bytes, kv->pool, pool_bytes))
     return fail(HAM_EINVAL, "q_inout, out, k_new, v_new and the cache must not overlap");
-  const int64_t blocks = (int64_t)total_rows / ham::prefill_query_rows(group) + c.batch;
-  if (blocks > 65535)
-    return fail(HAM_EINVAL, "total_rows %d: split the chunk (at most %lld query blocks a call)",
-                total_rows, 65535LL);
+  const int64_t blocks = ham::prefill_blocks(total_rows, c.batch, ham::prefill_query_rows(group));
+  if (blocks > ham::kPrefillMaxBlocks)
+    return fail(HAM_EINVAL, "total_rows %d: split the chunk (at most %d query blocks a call)",
+                total_rows, ham::kPrefillMaxBlocks);
   DeviceGuard guard(kv->device);
   ham::PrefillView v{};
   v.k_pool = layer_pool(kv, layer, 0);
@@ -1087,6 +1108,10 @@ int ham_prefill(ham_kv *kv, int32_t layer, void *q_inout, const void *k_new, con
     v.part_o = kv->prefill_part;
     v.part_ml = kv->prefill_part_ml;
   }
+  v.blocks = (int32_t)blocks;
+  v.next_item = kv->prefill_next;
+  v.order = kv->prefill_order;
+  v.sms = kv->num_sms;
   v.err = kv->err;
   v.pool_pages = c.pool_pages;
   v.batch = c.batch;
@@ -1098,8 +1123,8 @@ int ham_prefill(ham_kv *kv, int32_t layer, void *q_inout, const void *k_new, con
   v.max_pages = kv->max_pages;
   v.max_slots = c.max_slots_per_seq;
   v.pos_mode = c.pos_mode;
-  cudaError_t e = ham::launch_prefill(kv->tmaps_half[(size_t)layer * 2],
-                                      kv->tmaps_half[(size_t)layer * 2 + 1], v, out_dtype,
+  cudaError_t e = ham::launch_prefill(kv->tmaps_group[(size_t)layer * 2],
+                                      kv->tmaps_group[(size_t)layer * 2 + 1], v, out_dtype,
                                       static_cast<cudaStream_t>(stream));
   if (e != cudaSuccess) return cuda_fail(e, "prefill launch");
   note_launch(kv, layer, stream, true);

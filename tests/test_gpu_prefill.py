@@ -75,8 +75,8 @@ def test_prefill_matches_oracle(hq, hkv, d, page, cached, rows):
     assert_parity(_out(out), ref, what="prefill output")
 
 
-# Short chunks over long caches: the attention grid is split over the cached slots (each split at
-# least 8 tiles of 64 cached slots) and a merge kernel combines the splits' partials; sequences
+# Short chunks over long caches: the attention's items are split over the cached slots (each split at
+# least 512 cached slots) and a merge kernel combines the splits' partials; sequences
 # with few cached slots in the same call stay whole.
 @pytest.mark.parametrize("hq,hkv,d,page,cached,rows,f32", [
     (32, 8, 128, 16, (4096, 1500), (40, 9), False),      # 8 and 2 splits; Llama-8B heads
@@ -95,6 +95,42 @@ def test_prefill_split_over_slots_matches_oracle(hq, hkv, d, page, cached, rows,
     assert ham.ham_kv_status(kv) == ham.HAM_DEVERR_NONE
     _check_state(kv, q, oc, q_ref)
     assert_parity(_out(out), ref, what="split prefill output" + (" (f32)" if f32 else ""))
+
+
+# The attention's tiles hold 128 slots in blocks of 64 and chunks of 16, and 128 / group query rows:
+# sizes at and beside every edge, more items than SMs, a block order over unequal chunks.
+@pytest.mark.parametrize("hq,hkv,d,cached,rows", [
+    (8, 2, 128, (0, 0, 0, 0), (1, 63, 64, 65)),
+    (8, 2, 64, (0, 0, 0, 0), (16, 31, 32, 33)),
+    (8, 2, 128, (64, 63, 127, 128), (64, 2, 1, 129)),
+    (8, 2, 64, (64, 63, 127, 128), (64, 2, 1, 129)),
+    (16, 2, 64, (112, 113, 0), (16, 17, 150)),           # group 8: 16-row Q tiles
+    (4, 4, 128, (48, 200), (257, 128)),                  # group 1: 128-row Q tiles
+    (32, 8, 128, (0, 300, 5, 70), (700, 333, 1, 450)),   # 192 items
+])
+def test_prefill_tile_edges(hq, hkv, d, cached, rows):
+    w = _w(len(rows), hq, hkv, d, 16, seed=sum(rows) + d)
+    case = wl.make_prefill_case(w, rows, cached=np.array(cached, np.int32))
+    kv, q, out = _gpu(case)
+    oc, q_ref, rc, ref = _oracle(case)
+    assert rc == 0
+    assert ham.ham_kv_status(kv) == ham.HAM_DEVERR_NONE
+    _check_state(kv, q, oc, q_ref)
+    assert_parity(_out(out), ref, what="prefill output")
+
+
+@pytest.mark.parametrize("d", [64, 128])
+def test_prefill_rising_maximum(d):
+    """Scores with a standard deviation of 16: the running maximum rises past 2^8 in many rows after
+    their first block, so O is rescaled in tensor memory.  Values four times as large as in the other
+    cases, and so is the bar (the error of a bf16 weight or result scales with the values)."""
+    w = _w(2, 8, 2, d, 16, seed=77 + d, scale=4.0)
+    case = wl.make_prefill_case(w, (150, 70), cached=np.array([500, 20], np.int32))
+    kv, q, out = _gpu(case, f32=True)
+    oc, q_ref, rc, ref = _oracle(case)
+    assert rc == 0
+    _check_state(kv, q, oc, q_ref)
+    assert_parity(_out(out), ref, max_abs=8e-2, mean_abs=8e-3, what="prefill output, rising maximum")
 
 
 @pytest.mark.parametrize("mode", ["token", "explicit"])
