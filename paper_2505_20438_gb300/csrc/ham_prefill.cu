@@ -100,6 +100,9 @@ __device__ __forceinline__ int block_scan(int x, int *red, int *total) {
 __global__ void __launch_bounds__(kPlanThreads) prefill_plan_kernel(PrefillView v, int qb_rows) {
   __shared__ int red[kPlanThreads / 32];
   const int b = blockIdx.x, tid = threadIdx.x, B = v.batch;
+  // The RoPE kernel may be scheduled now: it reads the call's inputs, and waits for this grid (which
+  // itself starts after everything before it on the stream) before it reads the plan or writes.
+  grid_launch_dependents();
   if (b == 0 && tid == 0) *v.next_item = 0;  // the attention's items are handed out from here
   // The offsets must describe the call's rows: every block checks all of them, so that all agree.
   int bad_off = 0;
@@ -284,14 +287,16 @@ __global__ void __launch_bounds__(kRopeThreads) prefill_rope_kernel(PrefillView 
     const uint16_t *src = h < Hq ? qrow + h * D : krow + (h - Hq) * D;
     return *reinterpret_cast<const uint4 *>(src + upper * kHalf + 8 * j);
   };
-  // 1. the loads (the row's pool row is -1 when it is not stored; the call's offsets are valid
-  //    when sequence 0's plan entry says so)
-  const int2 ri = v.row_info[r];
-  const int offsets_ok = v.seq_info[0].w;
+  // 1. the loads: the call's inputs, then what the plan left (the row's pool row is -1 when it is
+  //    not stored; the call's offsets are valid when sequence 0's plan entry says so)
   uint4 x0l{}, x0h{}, x1l{}, x1h{}, vv{};
   if (h0 < H) { x0l = half_of(h0, 0); x0h = half_of(h0, 1); }
   if (h1 < H) { x1l = half_of(h1, 0); x1h = half_of(h1, 1); }
   if (tid < nv) vv = vrow[tid];
+  grid_dependency_wait();
+  grid_launch_dependents();  // the attention may be scheduled as this grid drains
+  const int2 ri = v.row_info[r];
+  const int offsets_ok = v.seq_info[0].w;
   const int p = ri.x;
   const bool in_table = p >= 0 && p < v.rope_positions;
   float4 c4{};
@@ -578,6 +583,8 @@ __global__ void __launch_bounds__(TcShape<D>::kThreads, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  grid_dependency_wait();  // the plan, the rotated queries and the stored rows
+  grid_launch_dependents();
   // ring and data waits: the launch's limit; item hand-over and the draining of in-flight work
   // keep the default 2 s
   const uint64_t wait_lim = data_wait_limit(v.wait_ns);
@@ -1012,13 +1019,18 @@ __global__ void __launch_bounds__(TcShape<D>::kThreads, 1)
 // out = sum_z 2^(m_z - M) O_z / sum_z 2^(m_z - M) l_z over the splits z of the row's sequence, in
 // split order (M = max_z m_z; the split-softmax merge of the decode combine).  One warp per
 // (row, head), D / 32 elements a lane; rows of sequences that were not split (written by the
-// attention itself) or that the plan refused are left alone.
-constexpr int kMergeWarps = 8;
-template <typename OutT>
+// attention itself) or that the plan refused are left alone.  Lane z takes split z's (max, sum) and
+// weight, and the partials are read kMergeBatch at a time: the kernel is bound by its round trips
+// to L2 (one split after the other took 18 us for 2,048 rows of 19 splits).
+constexpr int kMergeWarps = 8, kMergeBatch = 8;
+static_assert(kPrefillMaxSplits <= 32, "one lane a split");
+template <int D, typename OutT>
 __global__ void __launch_bounds__(kMergeWarps * 32) prefill_merge_kernel(const PrefillView v) {
+  constexpr int kPer = D / 32;  // elements a lane
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int Hq = v.n_q_heads, D = v.head_dim;
+  const int Hq = v.n_q_heads;
   const int64_t rh = (int64_t)blockIdx.x * kMergeWarps + warp;  // (row, head)
+  grid_dependency_wait();
   if (rh >= (int64_t)v.rows * Hq) return;
   const int r = (int)(rh / Hq);
   int lo = 0, hi = v.batch - 1;  // the row's sequence: the last b with offsets[b] <= r
@@ -1031,25 +1043,65 @@ __global__ void __launch_bounds__(kMergeWarps * 32) prefill_merge_kernel(const P
   const int zs = prefill_splits(si.x, v.splits);
   if (zs <= 1) return;
   const int64_t zstride = (int64_t)v.rows * Hq;
-  float M = -INFINITY;
-  for (int z = 0; z < zs; ++z) M = fmaxf(M, v.part_ml[z * zstride + rh].x);
-  const int per = D / 32;  // 4 or 2
-  float num[4] = {0.f, 0.f, 0.f, 0.f}, den = 0.f;
-  for (int z = 0; z < zs; ++z) {
-    const float2 ml = v.part_ml[z * zstride + rh];
-    const float w = ml.x == -INFINITY ? 0.f : ex2(ml.x - M);
-    den += w * ml.y;
-    const float *po = v.part_o + (z * zstride + rh) * D + lane * per;
-    for (int e = 0; e < per; ++e) num[e] += w * po[e];
+  const float2 ml = lane < zs ? v.part_ml[lane * zstride + rh] : make_float2(-INFINITY, 0.f);
+  const float M = warp_max_f32(ml.x);
+  const float w = ml.x == -INFINITY ? 0.f : ex2(ml.x - M);
+  float num[kPer], den = 0.f;
+#pragma unroll
+  for (int e = 0; e < kPer; ++e) num[e] = 0.f;
+  const float *po = v.part_o + rh * D + lane * kPer;
+  for (int z0 = 0; z0 < zs; z0 += kMergeBatch) {
+    float o[kMergeBatch][kPer];
+#pragma unroll
+    for (int x = 0; x < kMergeBatch; ++x) {
+      const float *src = po + (int64_t)min(z0 + x, zs - 1) * zstride * D;
+      if constexpr (kPer == 4) {
+        const float4 y = *reinterpret_cast<const float4 *>(src);
+        o[x][0] = y.x; o[x][1] = y.y; o[x][2] = y.z; o[x][3] = y.w;
+      } else {
+        const float2 y = *reinterpret_cast<const float2 *>(src);
+        o[x][0] = y.x; o[x][1] = y.y;
+      }
+    }
+#pragma unroll
+    for (int x = 0; x < kMergeBatch; ++x) {
+      const int z = z0 + x;
+      const float wz = __shfl_sync(kFull, w, z & 31), lz = __shfl_sync(kFull, ml.y, z & 31);
+      if (z < zs) {
+        den += wz * lz;
+#pragma unroll
+        for (int e = 0; e < kPer; ++e) num[e] += wz * o[x][e];
+      }
+    }
   }
   const float inv = den > 0.f ? 1.f / den : 0.f;
-  OutT *dst = static_cast<OutT *>(v.out) + rh * D + lane * per;
-  for (int e = 0; e < per; ++e) {
+  OutT *dst = static_cast<OutT *>(v.out) + rh * D + lane * kPer;
+#pragma unroll
+  for (int e = 0; e < kPer; ++e) {
     if constexpr (std::is_same<OutT, float>::value)
       dst[e] = num[e] * inv;
     else
       dst[e] = __float2bfloat16_rn(num[e] * inv);
   }
+}
+
+// A launch with programmatic dependent launch: the kernel may start before its predecessor on the
+// stream ends and waits for it (griddepcontrol.wait) before it reads or writes anything that the
+// predecessor writes or reads.
+template <typename... KArgs, typename... Args>
+cudaError_t launch_dependent(void (*kernel)(KArgs...), unsigned grid, int threads, size_t smem,
+                             cudaStream_t stream, const Args &...args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
 template <int D, typename OutT>
@@ -1061,13 +1113,13 @@ cudaError_t launch_attn(const CUtensorMap &tq, const CUtensorMap &tk, const CUte
   if (e != cudaSuccess) return e;
   const int64_t items = (int64_t)v.n_kv_heads * v.blocks * v.splits;
   const unsigned grid = (unsigned)(items < v.sms ? items : v.sms);  // persistent: one CTA an SM
-  prefill_attn_kernel<D, OutT><<<grid, S::kThreads, S::kSmem, stream>>>(tq, tk, tv, v);
-  e = cudaGetLastError();
+  e = launch_dependent(prefill_attn_kernel<D, OutT>, grid, S::kThreads, S::kSmem, stream, tq, tk,
+                       tv, v);
   if (e != cudaSuccess || v.splits == 1) return e;
   const int64_t pairs = (int64_t)v.rows * v.n_q_heads;
-  prefill_merge_kernel<OutT><<<(unsigned)((pairs + kMergeWarps - 1) / kMergeWarps),
-                               kMergeWarps * 32, 0, stream>>>(v);
-  return cudaGetLastError();
+  return launch_dependent(prefill_merge_kernel<D, OutT>,
+                          (unsigned)((pairs + kMergeWarps - 1) / kMergeWarps), kMergeWarps * 32, 0,
+                          stream, v);
 }
 
 template <typename OutT>
@@ -1080,11 +1132,9 @@ cudaError_t launch_all(const CUtensorMap &tk, const CUtensorMap &tv, const Prefi
   prefill_plan_kernel<<<(unsigned)v.batch, kPlanThreads, 0, stream>>>(v, prefill_query_rows(G));
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  if (v.head_dim == 128)
-    prefill_rope_kernel<128, OutT><<<(unsigned)v.rows, kRopeThreads, 0, stream>>>(v);
-  else
-    prefill_rope_kernel<64, OutT><<<(unsigned)v.rows, kRopeThreads, 0, stream>>>(v);
-  e = cudaGetLastError();
+  e = launch_dependent(v.head_dim == 128 ? prefill_rope_kernel<128, OutT>
+                                         : prefill_rope_kernel<64, OutT>,
+                       (unsigned)v.rows, kRopeThreads, 0, stream, v);
   if (e != cudaSuccess) return e;
   return v.head_dim == 128 ? launch_attn<128, OutT>(tq, tk, tv, v, stream)
                            : launch_attn<64, OutT>(tq, tk, tv, v, stream);
