@@ -32,6 +32,8 @@ struct MicroView {
   int64_t pool_pages;
   int32_t batch, n_q_heads, n_kv_heads, head_dim, page_slots, max_pages, max_slots, pos_mode;
   int32_t out_f32;
+  int32_t early;               // 1: the library state may be read before the dependency wait (as in
+                               // AttnView)
 };
 
 cudaError_t launch_micro(const MicroView &v, cudaStream_t stream);

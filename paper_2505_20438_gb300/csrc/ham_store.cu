@@ -1028,6 +1028,7 @@ int ham_micro_step(ham_kv *kv, int32_t layer, const void *q, void *q_rot, const 
   v.max_slots = c.max_slots_per_seq;
   v.pos_mode = c.pos_mode;
   v.out_f32 = out_dtype == HAM_DTYPE_F32 ? 1 : 0;
+  v.early = may_start_early(kv, layer, stream) ? 1 : 0;
   cudaError_t e = ham::launch_micro(v, static_cast<cudaStream_t>(stream));
   if (e != cudaSuccess) return cuda_fail(e, "micro step launch");
   note_launch(kv, layer, stream, true);

@@ -139,6 +139,47 @@ def test_micro_step_equals_decode_step():
         assert np.array_equal(x, y)
 
 
+@pytest.mark.parametrize("order", [(0, 1, 2), (0, 0, 1, 1, 1), (2, 0, 2, 1)])
+@pytest.mark.parametrize("d", [64, 128])
+def test_micro_step_layers_back_to_back(order, d):
+    """Launches with nothing between them, layers in turn (library state read before the launch
+    before has finished) and one layer repeated (read after it): every layer's bits, counters and
+    outputs as the oracle's."""
+    import torch
+    case = small_case(batch=4, hq=16, hkv=4, d=d, page=16, counts=(0, 1, 5, 7), seed=21 + d,
+                      extra_slots=9)
+    kv = gpu_cache(case, layers=3)
+    caches = [oracle.OracleCache.from_case(case) for _ in range(3)]
+    rng = wl.rng_for(21, d)
+    calls = []
+    weights = [wl.ntok_capped_geometric(rng, (4,)) for _ in range(9)]   # shared by the layers
+    seen = [0, 0, 0]
+    for layer in order * 3:
+        q = wl.normal_bf16(rng, (4, 16, d))
+        k_new = wl.normal_bf16(rng, (4, 4, d))
+        v_new = wl.normal_bf16(rng, (4, 4, d))
+        ntok = weights[seen[layer]]
+        seen[layer] += 1
+        calls.append((layer, q, k_new, v_new, ntok, dev_bf16(q), dev_bf16(k_new),
+                      dev_bf16(v_new), dev_i32(ntok),
+                      torch.full((4, 16, d), float("nan"), dtype=torch.float32, device="cuda")))
+    torch.cuda.synchronize()
+    for layer, _, _, _, _, q, k_new, v_new, ntok, out in calls:
+        ham.ham_micro_step(kv, layer, q, k_new, v_new, None, ntok, out)
+    torch.cuda.synchronize()
+    for i, (layer, q, k_new, v_new, ntok, *_, out) in enumerate(calls):
+        assert caches[layer].append(k_new, v_new, ntok, q_inout=q,
+                                    pos_mode=ham.HAM_POS_SLOT) == 0
+        assert_parity(out.cpu().numpy().astype(np.float64), caches[layer].decode_attn(q),
+                      F32_MAX_ABS, F32_MEAN_ABS, what=f"call {i}, layer {layer}")
+    for layer, oc in enumerate(caches):
+        k, v, p, n = _export(kv, layer)
+        assert np.array_equal(k, oc.k_pool) and np.array_equal(v, oc.v_pool)
+        if seen[layer] == max(seen):       # (positions and weights are shared by the layers)
+            assert np.array_equal(p, oc.slot_pos) and np.array_equal(n, oc.slot_ntok)
+    assert ham.ham_kv_status(kv) == ham.HAM_DEVERR_NONE
+
+
 def test_micro_step_failures():
     """A full sequence and ntok < 1: no slot, the error word set, attention with the unrotated
     query over the old slots; the other sequences proceed."""
