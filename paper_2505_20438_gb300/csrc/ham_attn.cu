@@ -582,8 +582,10 @@ __global__ void __launch_bounds__(Shape<D>::kThreads)
 // CTAs k = first..last of the segment, M = max_k m_k (split-softmax merge, in CTA order, in
 // batches of kBatch partials whose loads are in flight together).  One thread per pair of
 // elements (h, i) and (h, i + D/2) of an output row: both share the head's (max, sum), and for
-// the fused step they are the pair that RoPE turns together.  Blocks of kCombineThreads cover
-// one segment's G*D/2 pairs (whole heads).
+// the fused step they are the pair that RoPE turns together.  Blocks cover kPairs of one
+// segment's G*D/2 pairs (whole heads).  The merge is bound by its chain of round trips to L2, not
+// by bytes: a thread reading 33 partials took 3.0 to 3.7 us (two batches of up to 32), four groups
+// reading 9 each 1.4 us.
 //
 // Fused step: the pass covered the stored slots; the appended slot enters here as one more
 // term of the merge: score q.k / sqrt(d) with q and the new key turned by the new position in
@@ -619,6 +621,7 @@ constexpr int kCombineThreads = 128;
 // slots, -1.5% and -4% at 8192; unconditionally it cost 18% on the 32-layer stack at batch 1
 // (4 chunks a CTA) and 1.5% at batch 4 x 65536 (215 chunks a CTA), hence the window.
 constexpr int kTriggerChunksMin = 16, kTriggerChunksMax = 128;
+constexpr int kCombineSplit = 4;  // thread groups of a block that share a segment's partials
 constexpr int kCombinePlanBatch = kCombineThreads;  // batches whose plan the combine computes
 static_assert(kCombineThreads % 64 == 0, "a block holds whole heads of head_dim 64 or 128");
 
@@ -768,22 +771,31 @@ __device__ __forceinline__ void merge_partials(const AttnView &v, int seg, int h
   }
 }
 
-template <typename OutT, bool kStep, int kBatch>
-__global__ void __launch_bounds__(kCombineThreads) combine_kernel(const AttnView v, int D,
-                                                                  int blocks_per_seg) {
+// A block holds kPairs pairs.  kSplit > 1 (few segments, each of many partials): kSplit groups of
+// kPairs threads, each merging its share of the partials, so that all of a segment's partials are
+// read in one or two round trips of short batches; group 0 does the rest and merges the groups in
+// order.
+template <typename OutT, bool kStep, int kBatch, int kPairs, int kSplit>
+__global__ void __launch_bounds__(kPairs *kSplit) combine_kernel(const AttnView v, int D,
+                                                                 int blocks_per_seg) {
+  constexpr int kThreads = kPairs * kSplit, kWarps = kThreads / 32;
+  static_assert(kPairs % 64 == 0 && kThreads >= kCombinePlanBatch, "whole heads; a thread a sequence");
   const int G = v.group, Hkv = v.n_kv_heads, half = D / 2, B = v.batch;
   const int seg = blockIdx.x / blocks_per_seg;
   const int part = blockIdx.x % blocks_per_seg;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int idx = part * kCombineThreads + tid;  // pair index within the segment
+  const int group = tid / kPairs;
+  const int idx = part * kPairs + tid % kPairs;  // pair index within the segment
   const bool active = idx < G * half;
+  const bool lead = active && (kSplit == 1 || group == 0);  // owns the pair (h, i)
   const int h = idx / half, i = idx - h * half;
   const int b = seg / Hkv, g = seg - b * Hkv;
   const int64_t orow = ((int64_t)seg * G + h) * D;  // row (b, g*G + h) of q / q_rot / out
   const StepArgs &st = v.step;
-  __shared__ int red[3][kCombineThreads / 32];
-  __shared__ float head_sum[kCombineThreads / 32];
-  __shared__ float fp8_red[kCombineThreads / 32];
+  __shared__ int red[3][kWarps];
+  __shared__ float head_sum[kWarps];
+  __shared__ float fp8_red[kWarps];
+  __shared__ float4 group_part[kSplit > 1 ? kSplit - 1 : 1][kSplit > 1 ? kPairs : 1];
   __shared__ int commit_all;  // fused step: this CTA commits every sequence
   const bool fp8 = v.kv_exp != nullptr;  // FP8 pools
 
@@ -812,7 +824,7 @@ __global__ void __launch_bounds__(kCombineThreads) combine_kernel(const AttnView
     __syncthreads();
     int T = 0, P = 0, N = 0;
 #pragma unroll
-    for (int w = 0; w < kCombineThreads / 32; ++w) {
+    for (int w = 0; w < kWarps; ++w) {
       T += red[0][w];
       P += red[1][w];
       N += red[2][w];
@@ -843,7 +855,7 @@ __global__ void __launch_bounds__(kCombineThreads) combine_kernel(const AttnView
   int cpage = -1;
   if constexpr (kStep) {
     uint16_t q0 = 0, q1 = 0, k0 = 0, k1 = 0;
-    if (active) {  // caller inputs: final once the attention grid started
+    if (lead) {  // caller inputs: final once the attention grid started
       q0 = v.q[orow + i];
       q1 = v.q[orow + i + half];
       k0 = st.k_new[(int64_t)seg * D + i];
@@ -856,7 +868,7 @@ __global__ void __launch_bounds__(kCombineThreads) combine_kernel(const AttnView
     float share = 0.f;
     PairTurn pt{};
     int page = -1;
-    if (rec.y == 0 && active) {
+    if (rec.y == 0 && lead) {
       const double2 cs = rope_cs(st, rec.z, half, i);
       pt = turn_pair(cs.x, cs.y, q0, q1, k0, k1);
       share = pt.share;
@@ -874,7 +886,7 @@ __global__ void __launch_bounds__(kCombineThreads) combine_kernel(const AttnView
       }
     }
     if (fp8) {  // encode the rows as the append does; the new slot's term takes the decoded ones
-      const bool mine = rec.y == 0 && active;
+      const bool mine = rec.y == 0 && lead;
       const Fp8Pair kp = fp8_encode_pair(mine ? bf16_bits_to_float(pt.kc0) : 0.f,
                                          mine ? bf16_bits_to_float(pt.kc1) : 0.f, half, fp8_red);
       const Fp8Pair vp = fp8_encode_pair(mine ? bf16_bits_to_float(v0) : 0.f,
@@ -916,12 +928,30 @@ __global__ void __launch_bounds__(kCombineThreads) combine_kernel(const AttnView
 
   const bool merge = first >= 0 && (kStep || first != last);
   float M = -INFINITY, num0 = 0.f, num1 = 0.f, den = 0.f;
-  if (active && merge)
-    merge_partials<kBatch>(v, seg, h, i, half, D, first, last, M, num0, num1, den);
+  if (active && merge) {
+    const int share = kSplit == 1 ? last - first + 1 : (last - first + kSplit) / kSplit;
+    const int lo = first + group * share;
+    merge_partials<kBatch>(v, seg, h, i, half, D, lo, min(last, lo + share - 1), M, num0, num1, den);
+  }
+  if constexpr (kSplit > 1) {
+    if (group > 0) group_part[group - 1][tid % kPairs] = make_float4(M, num0, num1, den);
+    __syncthreads();
+#pragma unroll
+    for (int x = 0; x < kSplit - 1; ++x) {
+      const float4 o = group_part[x][tid % kPairs];
+      const float bm = fmaxf(M, o.x);
+      const float a = (M == -INFINITY) ? 0.f : ex2(M - bm);
+      const float c = (o.x == -INFINITY) ? 0.f : ex2(o.x - bm);
+      num0 = num0 * a + c * o.y;
+      num1 = num1 * a + c * o.z;
+      den = den * a + c * o.w;
+      M = bm;
+    }
+  }
 
   if constexpr (kStep) {
     const bool appended = rec.y == 0;
-    if (appended && active) {  // the appended slot: one more term of the merge
+    if (appended && lead) {  // the appended slot: one more term of the merge
       const float x = dot * (rsqrtf((float)D) * 1.4426950408889634f);  // log2 domain
       const float bm = fmaxf(M, x);
       const float scale = (M == -INFINITY) ? 0.f : ex2(M - bm);
@@ -930,7 +960,7 @@ __global__ void __launch_bounds__(kCombineThreads) combine_kernel(const AttnView
       num1 = num1 * scale + w * (fp8 ? vd1 : bf16_bits_to_float(v1));
       den = den * scale + w;
     }
-    if (active && (merge || appended)) {
+    if (lead && (merge || appended)) {
       const float inv = den > 0.f ? 1.f / den : 0.f;
       store_out<OutT>(v.out, orow + i, num0 * inv);
       store_out<OutT>(v.out, orow + i + half, num1 * inv);
@@ -952,7 +982,7 @@ __global__ void __launch_bounds__(kCombineThreads) combine_kernel(const AttnView
     st.num_slots[tid] = crec.x + 1;
     st.num_tokens[tid] = ctok + crec.w;
   } else {
-    if (active && merge) {
+    if (lead && merge) {
       const float inv = den > 0.f ? 1.f / den : 0.f;  // 0: every slot masked
       store_out<OutT>(v.out, orow + i, num0 * inv);
       store_out<OutT>(v.out, orow + i + half, num1 * inv);
@@ -1130,14 +1160,16 @@ inline bool combine_early(const AttnView &v, int64_t combine_ctas, bool step) {
   return v.batch <= kCombinePlanBatch && (!step || combine_ctas <= (int64_t)v.sms);
 }
 
-// Early mode's merge batch: a segment spans about ctas / segments + 1 CTAs when the lengths
-// are equal, and 32 or 16 partials in flight save round trips when there are that many.
+// Early mode's merge: a segment spans about ctas / segments + 1 CTAs when the lengths are equal.
+// From 24 partials a segment on, a block of 64 pairs shares them among kCombineSplit groups of
+// threads (33 partials, one sequence of 2048 slots: 8.5 us a step against 10.6 with one thread reading
+// 32 at a time), as long as these smaller blocks still sit beside the pass; 16 in flight save round
+// trips from 7 on.
 template <typename OutT, bool kStep>
 cudaError_t launch_combine(const AttnView &v, int head_dim, cudaStream_t stream) {
-  const int per_seg = (v.group * head_dim / 2 + kCombineThreads - 1) / kCombineThreads;
+  const int pairs = v.group * head_dim / 2;
   const int64_t segs = (int64_t)v.batch * v.n_kv_heads;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(segs * per_seg));
   cfg.blockDim = dim3(kCombineThreads);
   cfg.stream = stream;
   cudaLaunchAttribute attr[1];
@@ -1145,13 +1177,22 @@ cudaError_t launch_combine(const AttnView &v, int head_dim, cudaStream_t stream)
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
+  const int small = (pairs + 63) / 64;
+  if ((int64_t)v.ctas >= 24 * segs && combine_early(v, segs * small, kStep)) {
+    cfg.gridDim = dim3((unsigned)(segs * small));
+    cfg.blockDim = dim3(64 * kCombineSplit);
+    return cudaLaunchKernelEx(&cfg, combine_kernel<OutT, kStep, 12, 64, kCombineSplit>, v, head_dim,
+                              small);
+  }
+  const int per_seg = (pairs + kCombineThreads - 1) / kCombineThreads;
+  cfg.gridDim = dim3((unsigned)(segs * per_seg));
   if (!combine_early(v, segs * per_seg, kStep))
     return cudaLaunchKernelEx(&cfg, combine_late_kernel<OutT, kStep>, v, head_dim, per_seg);
-  if ((int64_t)v.ctas >= 24 * segs)
-    return cudaLaunchKernelEx(&cfg, combine_kernel<OutT, kStep, 32>, v, head_dim, per_seg);
   if ((int64_t)v.ctas >= 7 * segs)
-    return cudaLaunchKernelEx(&cfg, combine_kernel<OutT, kStep, 16>, v, head_dim, per_seg);
-  return cudaLaunchKernelEx(&cfg, combine_kernel<OutT, kStep, 8>, v, head_dim, per_seg);
+    return cudaLaunchKernelEx(&cfg, combine_kernel<OutT, kStep, 16, kCombineThreads, 1>, v, head_dim,
+                              per_seg);
+  return cudaLaunchKernelEx(&cfg, combine_kernel<OutT, kStep, 8, kCombineThreads, 1>, v, head_dim,
+                            per_seg);
 }
 
 // ------------------------------------------------------------------------------------

@@ -12,7 +12,7 @@ from paper_2505_20438_gb300 import ham
 from paper_2505_20438_gb300 import workload as wl
 
 from gpu_helpers import (MAX_ABS, MEAN_ABS, assert_parity, dev_bf16, dev_i32, gpu_cache,
-                         host_bits, small_case, torch)
+                         gpu_decode, host_bits, small_case, torch)
 
 pytestmark = pytest.mark.gpu
 
@@ -162,6 +162,25 @@ def test_step_split_counts(ctas):
     got, q_rot = _step(kv, case.q, case.k_new, case.v_new, case.ntok_new)
     assert np.array_equal(q_rot, q_ref)
     assert_parity(got, oc.decode_attn(q_ref), MAX_ABS, MEAN_ABS, what=f"ctas={ctas}")
+    _assert_cache_equal(kv, oc)
+
+
+@pytest.mark.parametrize("d,hq,hkv", [(128, 8, 1), (128, 1, 1), (128, 12, 4), (64, 4, 2), (64, 1, 1)])
+@pytest.mark.parametrize("counts", [(1,), (63,), (64, 65), (2047,), (2048 + 17, 5, 0), (9000,)])
+def test_step_shared_merge(d, hq, hkv, counts):
+    """Few segments: a block's thread groups share a segment's partials (none, fewer than groups,
+    uneven shares, several batches), for the fused step and the attention alone.  fp32 merging as
+    before, so the bar is the decode one."""
+    case = small_case(batch=len(counts), hq=hq, hkv=hkv, d=d, page=16, counts=counts,
+                      seed=d + hq + sum(counts), extra_slots=4)
+    oc = oracle.OracleCache.from_case(case)
+    kv = gpu_cache(case)
+    assert_parity(gpu_decode(kv, case.q, f32=True), oc.decode_attn(case.q), what="attention")
+    q_ref = case.q.copy()
+    assert oc.append(case.k_new, case.v_new, case.ntok_new, q_inout=q_ref) == 0
+    got, q_rot = _step(kv, case.q, case.k_new, case.v_new, case.ntok_new)
+    assert np.array_equal(q_rot, q_ref)
+    assert_parity(got, oc.decode_attn(q_ref), what="step")
     _assert_cache_equal(kv, oc)
 
 
