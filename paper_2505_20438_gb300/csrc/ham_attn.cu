@@ -58,6 +58,8 @@ struct Shape {
   static constexpr int kStages = 32768 / kStageBytes;       // 32 KiB ring
   static constexpr int kQBufs = kStages + 1;
   static constexpr int kThreads = 64;                       // consumer warp, producer warp
+  // At most 128 registers: four CTAs, a combine block and the next pass's first CTA fit an SM.
+  static constexpr int kRegBlocks = 65536 / (128 * kThreads);
   static constexpr int kSteps = D / 16;                     // k-steps of q.k, m-tiles of p.v
   static constexpr int kLinesPerRow = D / 64;               // 128-byte swizzle lines per row
   static constexpr int kOffQ = kStages * kStageBytes;       // from a 1024-byte aligned base
@@ -119,7 +121,7 @@ __device__ __forceinline__ uint16_t rotate_elem(double self, double other, doubl
 // The kernel
 // ------------------------------------------------------------------------------------
 template <int D, typename OutT, bool kStep>
-__global__ void __launch_bounds__(Shape<D>::kThreads)
+__global__ void __launch_bounds__(Shape<D>::kThreads, Shape<D>::kRegBlocks)
     decode_attn_kernel(const __grid_constant__ CUtensorMap tmap_k,
                        const __grid_constant__ CUtensorMap tmap_v, const AttnView v) {
   using S = Shape<D>;
@@ -229,26 +231,52 @@ __global__ void __launch_bounds__(Shape<D>::kThreads)
          ((c == nch - 1 || x == x1 - 1) ? kLast : 0);
   };
 
-  // The first ring's worth of K/V copies.  Their stages expect the K/V bytes now and arrive
-  // (with the bytes of q and the step rows, if the stage opens a segment) after the wait.
+  // The first ring's stages.  A stage that opens no segment needs nothing of the caller: it is
+  // described and armed now.  One that does (`opens`) gets its K/V copies now, the segment's
+  // (cos, sin) row too where the position is library state, and q and its arrival after the wait.
+  // (Per step, with the combine's earlier trigger and loads, against arming every stage after the
+  // wait: one sequence of 2048 slots 8.14 us and 8.54; 8 x 2048 16.8 and 17.5, head_dim 64 13.1 and
+  // 14.7; 8 x 200 8.9 and 9.9.)
   int seg0 = 0, valid0 = 0, fl0 = 0, row00 = 0, pre = 0;
+  uint32_t opens = 0;
+  const bool given_pos = kStep && v.step.pos != nullptr;
+  auto load_cs_row = [&](int stage, int qb, int b) {  // (cos, sin) of the new slot's position
+    const int64_t p = posb[b];
+    if (p < 0 || p >= v.step.rope_positions) return;
+    mbar_expect_tx(&full[stage], (uint32_t)(D / 2) * 8);
+    bulk_load(qbufs + qb * sb.stride + sb.cs_off(), v.step.rope_table_f + p * (D / 2), (D / 2) * 8,
+              &full[stage]);
+  };
   if (warp == 1 && active_cta) {
     const int nb = min(32, nchunks);
     if (lane < nb) decode(0, seg0, valid0, fl0, row00);
     pre = min(nb, S::kStages);
+    opens = __ballot_sync(kFull, lane < pre && (fl0 & kFirst));
     const uint64_t pol = policy_evict_first();
     // The first segment's q into L2 while the previous kernel ends (a prefetch reads nothing
     // into the CTA: the copy below, after the dependency wait, takes q as that kernel left it)
     if (early && lane == 0 && nb > 0)
       bulk_prefetch_l2(v.q + (int64_t)seg0 * G * D, (uint32_t)sb.q_bytes);  // lane 0: chunk 0
     for (int j = 0; j < pre; ++j) {
+      const int s_seg = __shfl_sync(kFull, seg0, j);
+      const int s_valid = __shfl_sync(kFull, valid0, j);
       const int s_fl = __shfl_sync(kFull, fl0, j);
       const int s_row = __shfl_sync(kFull, row00, j);
-      if (lane == 0 && (s_fl & kPageOk)) {
-        uint8_t *dst = stages + j * S::kStageBytes;
-        mbar_expect_tx(&full[j], (uint32_t)S::kStageBytes);
-        tma_load_3d(dst, &tmap_k, 0, 0, s_row, &full[j], pol);
-        tma_load_3d(dst + S::kChunkBytes, &tmap_v, 0, 0, s_row, &full[j], pol);
+      if (lane == 0) {
+        const int qb = (s_fl & kFirst) ? __popc(opens & ((1u << j) - 1)) : -1;
+        info[j] = make_int4(s_seg, s_valid, s_fl, qb);
+        if (s_fl & kPageOk) {
+          uint8_t *dst = stages + j * S::kStageBytes;
+          if (qb < 0) mbar_arrive_tx(&full[j], (uint32_t)S::kStageBytes);
+          else mbar_expect_tx(&full[j], (uint32_t)S::kStageBytes);
+          tma_load_3d(dst, &tmap_k, 0, 0, s_row, &full[j], pol);
+          tma_load_3d(dst + S::kChunkBytes, &tmap_v, 0, 0, s_row, &full[j], pol);
+        } else {
+          record_error(v.err, HAM_DEVERR_PAGE);
+          if (qb < 0) mbar_arrive(&full[j]);
+        }
+        if constexpr (kStep)
+          if (qb >= 0 && !given_pos) load_cs_row(j, qb, s_seg / Hkv);
       }
     }
   }
@@ -256,11 +284,18 @@ __global__ void __launch_bounds__(Shape<D>::kThreads)
     grid_dependency_wait();
     grid_launch_dependents();
   }
-  // The first segment's q (buffer 0, stage 0): its copy needs nothing of what warp 0 reads
-  // next, so it is under way meanwhile.
-  if (warp == 1 && active_cta && lane == 0) {
-    mbar_expect_tx(&full[0], (uint32_t)sb.q_bytes);
-    bulk_load(qbufs, v.q + (int64_t)seg0 * G * D, (uint32_t)sb.q_bytes, &full[0]);
+  // The q heads of the first ring's segments (stages in order, buffers 0, 1, ...): their copies
+  // need nothing of what warp 0 reads next, so they are under way meanwhile.
+  if (warp == 1 && active_cta) {
+    int qb = 0;
+    for (uint32_t m = opens; m; m &= m - 1, ++qb) {
+      const int j = __ffs(m) - 1, s_seg = __shfl_sync(kFull, seg0, j);
+      if (lane == 0) {
+        if (given_pos) mbar_expect_tx(&full[j], (uint32_t)sb.q_bytes);
+        else mbar_arrive_tx(&full[j], (uint32_t)sb.q_bytes);
+        bulk_load(qbufs + qb * sb.stride, v.q + (int64_t)s_seg * G * D, (uint32_t)sb.q_bytes, &full[j]);
+      }
+    }
   }
   if constexpr (kStep) {
     // Caller inputs of the append: explicit positions, and whether each append happens.
@@ -300,61 +335,54 @@ __global__ void __launch_bounds__(Shape<D>::kThreads)
   // ---------------------------------------------------------------- producer warp
   if (warp == 1) {
     const uint64_t pol = policy_evict_first();
-    int it = 0, nseg = 0;
+    int it = pre, nseg = __popc(opens);
+    if (given_pos) {  // the first ring's remaining arrivals, now that the positions are known
+      int qb = 0;
+      for (uint32_t m = opens; m; m &= m - 1, ++qb) {
+        const int j = __ffs(m) - 1, s_seg = __shfl_sync(kFull, seg0, j);
+        if (lane == 0) {
+          if constexpr (kStep) load_cs_row(j, qb, s_seg / Hkv);
+          mbar_arrive(&full[j]);
+        }
+      }
+    }
     for (int base = 0; base < nchunks; base += 32) {
       const int nb = min(32, nchunks - base);
       int seg = seg0, valid = valid0, fl = fl0, row0 = row00;
       if (base > 0 && lane < nb) decode(base, seg, valid, fl, row0);
       bool stop = false;
-      for (int j = 0; j < nb; ++j) {
+      for (int j = base > 0 ? 0 : pre; j < nb; ++j) {
         const int s_seg = __shfl_sync(kFull, seg, j);
         const int s_valid = __shfl_sync(kFull, valid, j);
         const int s_fl = __shfl_sync(kFull, fl, j);
         const int s_row = __shfl_sync(kFull, row0, j);
-        const bool issued = it < pre;  // K/V already on their way (first ring)
         int failed = 0;
         if (lane == 0) {
           const int stage = it % S::kStages;
           const uint32_t ph = (uint32_t)(it / S::kStages) & 1u;
-          if (!issued && !thread_wait(&empty[stage], ph ^ 1u, flags, true, wait_lim)) {
+          if (!thread_wait(&empty[stage], ph ^ 1u, flags, true, wait_lim)) {
             record_error(v.err, HAM_DEVERR_TIMEOUT);
             flags[0] = 1;
             failed = 1;
           } else {
             int qb = -1;
-            bool tabled = false;
-            const int b = s_seg / Hkv;
             if (s_fl & kFirst) qb = nseg++ % S::kQBufs;
             info[stage] = make_int4(s_seg, s_valid, s_fl, qb);
-            uint32_t bytes = ((s_fl & kPageOk) && !issued) ? (uint32_t)S::kStageBytes : 0u;
-            if (qb >= 0) {
-              if (it > 0) bytes += (uint32_t)sb.q_bytes;  // (the first one is on its way)
-              if constexpr (kStep) {
-                const int64_t p = posb[b];
-                tabled = p >= 0 && p < v.step.rope_positions;
-                bytes += tabled ? (uint32_t)(D / 2) * 8 : 0u;
-              }
-            }
-            if (bytes) mbar_arrive_tx(&full[stage], bytes);
-            else mbar_arrive(&full[stage]);
             uint8_t *dst = stages + stage * S::kStageBytes;
-            if (!(s_fl & kPageOk)) {
-              record_error(v.err, HAM_DEVERR_PAGE);
-            } else if (!issued) {
+            if (s_fl & kPageOk) {
+              mbar_expect_tx(&full[stage], (uint32_t)S::kStageBytes);
               tma_load_3d(dst, &tmap_k, 0, 0, s_row, &full[stage], pol);
               tma_load_3d(dst + S::kChunkBytes, &tmap_v, 0, 0, s_row, &full[stage], pol);
+            } else {
+              record_error(v.err, HAM_DEVERR_PAGE);
             }
             if (qb >= 0) {
-              uint8_t *qdst = qbufs + qb * sb.stride;
-              if (it > 0)
-                bulk_load(qdst, v.q + (int64_t)s_seg * G * D, (uint32_t)sb.q_bytes, &full[stage]);
-              if constexpr (kStep) {  // (cos, sin) of the new slot's position
-                if (tabled)
-                  bulk_load(qdst + sb.cs_off(),
-                            v.step.rope_table_f + (int64_t)posb[b] * (D / 2), (D / 2) * 8,
-                            &full[stage]);
-              }
+              mbar_expect_tx(&full[stage], (uint32_t)sb.q_bytes);
+              bulk_load(qbufs + qb * sb.stride, v.q + (int64_t)s_seg * G * D, (uint32_t)sb.q_bytes,
+                        &full[stage]);
+              if constexpr (kStep) load_cs_row(stage, qb, s_seg / Hkv);
             }
+            mbar_arrive(&full[stage]);
           }
         }
         if (__shfl_sync(kFull, failed, 0)) {
@@ -611,15 +639,18 @@ __global__ void __launch_bounds__(Shape<D>::kThreads)
 // the CTAs that start after it would do the early work on the critical path.)
 // ------------------------------------------------------------------------------------
 constexpr int kCombineThreads = 128;
-// Early mode: when the pass gives its CTAs 16 to 128 chunks each, combine_kernel lets the next
-// kernel be scheduled at its start instead of after its wait.  The next attention grid's CTAs
-// then take the SM slots that this pass's CTAs free (and the spare one) and plan and prefetch
-// while this pass ends; their dependency wait still covers this grid, and what they read before
-// it is as before (state the immediately preceding kernel does not write; this pass, two
-// launches back, writes only its own handle's scratch and outputs, which a following kernel
-// touches only after its wait).  Measured per step: -2.6% (bf16) and -7% (FP8) at batch 8 x 4096
-// slots, -1.5% and -4% at 8192; unconditionally it cost 18% on the 32-layer stack at batch 1
-// (4 chunks a CTA) and 1.5% at batch 4 x 65536 (215 chunks a CTA), hence the window.
+// Early mode: combine_kernel lets the next kernel be scheduled before its own wait: at its start
+// when the pass gives its CTAs 16 to 128 chunks each, once its work before the wait is done when it
+// gives them fewer.
+// The next attention grid's CTAs then take the SM slots that this pass's CTAs free (and the spare
+// one) and plan and prefetch while this pass ends; their dependency wait still covers this grid, and
+// what they read before it is as before (state the immediately preceding kernel does not write;
+// this pass, two launches back, writes only its own handle's scratch and outputs, which a following
+// kernel touches only after its wait).  Measured per step: at the start against after the wait
+// -2.6% (bf16) and -7% (FP8) at batch 8 x 4096 slots, -1.5% and -4% at 8192; below that
+// window it cost 2.5% (batch 1 x 16384) to 4% (8 x 200) against just before the wait, which gave
+// -10% at 8 x 200 and -9% at 1 x 300 against after it; above (batch 4 x 65536, 215 chunks a CTA)
+// either costs 1.2%, so the trigger stays after the wait there.
 constexpr int kTriggerChunksMin = 16, kTriggerChunksMax = 128;
 constexpr int kCombineSplit = 4;  // thread groups of a block that share a segment's partials
 constexpr int kCombinePlanBatch = kCombineThreads;  // batches whose plan the combine computes
@@ -801,10 +832,26 @@ __global__ void __launch_bounds__(kPairs *kSplit) combine_kernel(const AttnView 
 
   // ---- the segment's CTA range (split plan, as the attention computes it)
   int first = -1, last = -1;
-  bool heavy = false;  // the same in every CTA
+  bool heavy = false, lengthy = false;  // the same in every CTA
   int Lt = 0;  // thread t < B: the slot counter of sequence t
+  int Lb = 0, tnew = 0;  // fused step: the segment's slot counter, the new slot's tokens
+  int64_t tb = 0;
+  uint16_t q0 = 0, q1 = 0, k0 = 0, k1 = 0, v0 = 0, v1 = 0;
   {
     int nch = 0;
+    if constexpr (kStep) {  // loads of the step, in the round trip of the plan's
+      Lb = v.num_slots[b];
+      if (!st.pos && st.pos_mode == HAM_POS_TOKEN) tb = st.num_tokens[b];
+      tnew = st.ntok[b];
+      if (lead) {  // caller inputs: final once the attention grid started
+        q0 = v.q[orow + i];
+        q1 = v.q[orow + i + half];
+        k0 = st.k_new[(int64_t)seg * D + i];
+        k1 = st.k_new[(int64_t)seg * D + i + half];
+        v0 = st.v_new[(int64_t)seg * D + i];
+        v1 = st.v_new[(int64_t)seg * D + i + half];
+      }
+    }
     if (tid < B) {
       Lt = v.num_slots[tid];
       nch = chunks_of(Lt < 0 ? 0 : (Lt > v.max_slots ? v.max_slots : Lt));
@@ -830,10 +877,11 @@ __global__ void __launch_bounds__(kPairs *kSplit) combine_kernel(const AttnView 
       N += red[2][w];
     }
     // A pass that streams kTriggerChunksMin..Max chunks a CTA lets the next kernel be scheduled
-    // now (see above); a shorter or a longer one keeps the trigger after the wait.
+    // now (see above), a shorter one just before the wait, a longer one after it.
     const int64_t Wt = (int64_t)Hkv * T;
     const int64_t Ct = plan_ctas(Wt, v.ctas);
-    heavy = Wt > 0 && Wt >= (int64_t)kTriggerChunksMin * Ct && Wt <= (int64_t)kTriggerChunksMax * Ct;
+    lengthy = Wt > (int64_t)kTriggerChunksMax * Ct;
+    heavy = Wt > 0 && Wt >= (int64_t)kTriggerChunksMin * Ct && !lengthy;
     if (N > 0) {
       const int64_t W = (int64_t)Hkv * T;
       const int C = plan_ctas(W, v.ctas);
@@ -845,26 +893,26 @@ __global__ void __launch_bounds__(kPairs *kSplit) combine_kernel(const AttnView 
 
   if (heavy) grid_launch_dependents();
 
-  // ---- fused step: record, rotations, q_rot and the new slot's rows; then the report
+  // ---- fused step: the report (every counter this CTA reads, but for the committing CTA's own,
+  // was read before the barrier above; no store is outstanding yet, so the fence is short); the
+  // record, rotations, q_rot and the new slot's rows
   int4 rec = make_int4(0, 0, 0, 0);
-  uint16_t v0 = 0, v1 = 0;
   float vd0 = 0.f, vd1 = 0.f;  // FP8 pools: the new value pair as the cache holds it
   float dot = 0.f;
   int4 crec = make_int4(0, 0, 0, 0);  // committing CTA, thread t < B: sequence t
   int64_t ctok = 0;
   int cpage = -1;
   if constexpr (kStep) {
-    uint16_t q0 = 0, q1 = 0, k0 = 0, k1 = 0;
-    if (lead) {  // caller inputs: final once the attention grid started
-      q0 = v.q[orow + i];
-      q1 = v.q[orow + i + half];
-      k0 = st.k_new[(int64_t)seg * D + i];
-      k1 = st.k_new[(int64_t)seg * D + i + half];
-      v0 = st.v_new[(int64_t)seg * D + i];
-      v1 = st.v_new[(int64_t)seg * D + i + half];
+    if (tid == kThreads - 1) {  // the last CTA to report commits every sequence
+      __threadfence();
+      const bool lastcta = atomicAdd(st.arrive, 1) == (int)gridDim.x - 1;
+      if (lastcta) {
+        *st.arrive = 0;
+        __threadfence();
+      }
+      commit_all = lastcta;
     }
-    const int64_t tb = (!st.pos && st.pos_mode == HAM_POS_TOKEN) ? st.num_tokens[b] : 0;
-    rec = append_record(v, v.num_slots[b], tb, st.ntok[b], st.pos ? st.pos + b : nullptr);
+    rec = append_record(v, Lb, tb, tnew, st.pos ? st.pos + b : nullptr);
     float share = 0.f;
     PairTurn pt{};
     int page = -1;
@@ -903,18 +951,8 @@ __global__ void __launch_bounds__(kPairs *kSplit) combine_kernel(const AttnView 
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) share += __shfl_xor_sync(kFull, share, off);
     if (lane == 0) head_sum[warp] = share;
-    __syncthreads();  // (also: every counter read of this CTA is consumed)
+    __syncthreads();  // (commit_all too)
     dot = half > 32 ? head_sum[warp & ~1] + head_sum[warp | 1] : head_sum[warp];
-    if (tid == 0) {  // report; the last CTA to report commits every sequence
-      __threadfence();
-      const bool lastcta = atomicAdd(st.arrive, 1) == (int)gridDim.x - 1;
-      if (lastcta) {
-        *st.arrive = 0;
-        __threadfence();
-      }
-      commit_all = lastcta;
-    }
-    __syncthreads();
     if (commit_all && tid < B) {  // its record, token count and page, while the pass runs
       ctok = st.num_tokens[tid];
       crec = append_record(v, Lt, ctok, st.ntok[tid], st.pos ? st.pos + tid : nullptr);
@@ -922,9 +960,10 @@ __global__ void __launch_bounds__(kPairs *kSplit) combine_kernel(const AttnView 
     }
   }
 
-  grid_dependency_wait();  // the attention grid's partials
   // The next kernel may be scheduled now; its own dependency wait still covers this grid.
-  if (!heavy) grid_launch_dependents();
+  if (!heavy && !lengthy) grid_launch_dependents();
+  grid_dependency_wait();  // the attention grid's partials
+  if (lengthy) grid_launch_dependents();
 
   const bool merge = first >= 0 && (kStep || first != last);
   float M = -INFINITY, num0 = 0.f, num1 = 0.f, den = 0.f;

@@ -165,6 +165,31 @@ def test_step_split_counts(ctas):
     _assert_cache_equal(kv, oc)
 
 
+@pytest.mark.parametrize("given", [False, True])
+@pytest.mark.parametrize("ctas", [1, 3])
+@pytest.mark.parametrize("d", [64, 128])
+def test_step_first_ring(d, ctas, given):
+    """Segments of one to three chunks, so that a CTA's first ring opens several: their stages are
+    armed before the wait or after it, with positions of the library and of the caller; two layers
+    in turn (read ahead of the wait), then one repeated."""
+    case = small_case(batch=4, hq=8, hkv=2, d=d, page=16, counts=(16, 1, 40, 0), seed=d + ctas,
+                      extra_slots=6)
+    oracles = [oracle.OracleCache.from_case(case) for _ in range(2)]
+    kv = gpu_cache(case, layers=2)
+    ham.ham_kv_set_attn_ctas(kv, ctas)
+    rng = wl.rng_for(d, ctas)
+    for i, layer in enumerate((0, 1, 0, 1, 1)):
+        q = wl.normal_bf16(rng, (4, 8, d))
+        k_new, v_new = wl.normal_bf16(rng, (4, 2, d)), wl.normal_bf16(rng, (4, 2, d))
+        pos = rng.integers(0, 9000, 4).astype(np.int32) if given else None
+        ntok = np.ones(4, np.int32)
+        q_ref = q.copy()
+        assert oracles[layer].append(k_new, v_new, ntok, q_inout=q_ref, pos=pos) == 0
+        got, q_rot = _step(kv, q, k_new, v_new, ntok, pos=pos, layer=layer)
+        assert np.array_equal(q_rot, q_ref)
+        assert_parity(got, oracles[layer].decode_attn(q_ref), what=f"call {i}")
+
+
 @pytest.mark.parametrize("d,hq,hkv", [(128, 8, 1), (128, 1, 1), (128, 12, 4), (64, 4, 2), (64, 1, 1)])
 @pytest.mark.parametrize("counts", [(1,), (63,), (64, 65), (2047,), (2048 + 17, 5, 0), (9000,)])
 def test_step_shared_merge(d, hq, hkv, counts):
