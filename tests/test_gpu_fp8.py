@@ -186,6 +186,17 @@ def test_decode_over_fp8_matches_oracle(hq, hkv, page, counts, scale):
     assert ham.ham_kv_status(kv) == ham.HAM_DEVERR_NONE
 
 
+@pytest.mark.parametrize("group", [1, 2, 5, 6, 7, 8])
+def test_decode_over_fp8_pairs_of_heads(group):
+    """Whole, partial and several tiles with every head of a pair, and an odd group's last head
+    alone (its partner masked), against the oracle at the fp32 bar."""
+    case = small_case(batch=3, hq=group, hkv=1, d=128, page=16, counts=(128, 17, 403),
+                      seed=group)
+    got = _decode(fp8_cache(case), case.q, f32=True)
+    assert_parity(got, _reference(case).decode_attn(case.q), max_abs=F32_MAX,
+                  mean_abs=F32_MEAN, what=f"group {group}")
+
+
 def test_decode_over_fp8_rows_of_very_different_scales():
     """Value rows whose scales differ by up to 2^40 across a sequence (the running value
     exponent is raised mid-segment and O rescaled), keys of mixed scales, and queries whose
