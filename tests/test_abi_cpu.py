@@ -221,3 +221,13 @@ def test_binding_rejects_host_tensors_without_a_handle():
     with pytest.raises(ValueError, match="k_pool must be a CUDA tensor"):
         ham.ham_decode_attn_noalloc(pool, pool, torch.zeros(2, 4, dtype=torch.int32),
                                     t["ntok"], t["q"], t["out"], 64)
+
+
+def test_binding_refuses_what_it_cannot_pass():
+    """The marshalling of tensors: none given, and a tensor of the host."""
+    import torch
+    assert ham._dev(None, (2,), "f32", "x", nullable=True) is None
+    with pytest.raises(ValueError, match="x is required"):
+        ham._dev(None, (2,), "f32", "x")
+    with pytest.raises(ValueError, match="must be a CUDA tensor"):
+        ham._dev(torch.zeros(2), (2,), "f32", "x")

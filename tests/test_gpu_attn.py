@@ -184,3 +184,20 @@ def test_full_size_workloads(w):
                       dev_i32(case.ntok_new))
     slots, _ = ham.ham_slot_lengths(kv)
     assert np.array_equal(slots, case.num_slots + 1)
+
+
+def test_binding_checks_and_streams():
+    """Tensors of another type, shape or layout are refused; the stream is the current one."""
+    import torch
+    x = torch.zeros((4, 6), device="cuda", dtype=torch.bfloat16)
+    assert ham._dev(x, (4, 6), "bf16", "x") == x.data_ptr()
+    for t, shape, dtype, why in ((x, (4, 6), "f32", "must be torch.float32"),
+                                 (x, (6, 4), "bf16", "must have shape"),
+                                 (x.t(), (6, 4), "bf16", "must be contiguous")):
+        with pytest.raises(ValueError, match=why):
+            ham._dev(t, shape, dtype, "x")
+    assert ham._stream_ptr(None) == torch.cuda.current_stream().cuda_stream
+    side = torch.cuda.Stream()
+    with torch.cuda.stream(side):
+        assert ham._stream_ptr(None) == side.cuda_stream
+    assert ham._stream_ptr(side) == side.cuda_stream and ham._stream_ptr(5) == 5
