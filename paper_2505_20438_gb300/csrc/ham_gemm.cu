@@ -16,8 +16,8 @@
 // through a TMA tensor map; X always through a tensor map (it is small and stays in L2); an X
 // stage always spans the 128 rows of the A layout, rows past the call's tile are never loaded
 // and only reach accumulator rows that are never stored.  Two MMA warps take alternate k-tiles
-// into two fp32 accumulators in tensor memory (one thread issues a tcgen05.mma only about
-// every 125 cycles, measured on GB300).  Eight epilogue warps (two a TMEM lane quarter, one
+// into two fp32 accumulators in tensor memory (a thread whose descriptors sit in its own registers
+// issues a tcgen05.mma only about every 100 to 125 cycles on GB300; the pipe takes one in 64).  Eight epilogue warps (two a TMEM lane quarter, one
 // half of the features each) add them: a thread holds 32 consecutive features of one row,
 // writes them into the (free) W ring in the 128-byte swizzle layout (no bank conflicts), and
 // each warp stores its 32 x 32 boxes with TMA (whole lines; the rows past the call clip at the

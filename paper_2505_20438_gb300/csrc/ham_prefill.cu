@@ -38,8 +38,8 @@
 //     Bound by each Q tile's chain scores -> softmax -> P V -> scores, which the other tile's
 //     covers in part: the tensor pipe is about 60% busy.  4 fresh prompts x 4096 rows of a
 //     Llama-8B layer, the whole call: 492 us, against 565 with 64-slot tiles, four issuing warps whose
-//     operands sat in per-thread registers and a CTA an item; 64 rows over 65,536 slots 93 against
-//     139 us; 4 x 2048 rows over 2048 slots at head_dim 64: 281 against 345.
+//     operands sat in per-thread registers and a CTA an item; 64 rows over 65,536 slots 80 against
+//     139 us (with the merge below); 4 x 2048 rows over 2048 slots at head_dim 64: 281 against 345.
 //  4. prefill_merge_kernel (split launches only), one warp per (row, head): the split-softmax
 //     merge of the partials in split order (as the decode combine merges its CTAs').
 //
