@@ -61,7 +61,7 @@ namespace {
 constexpr int kPlanThreads = 256;
 constexpr int kPlanRun = 8;  // consecutive rows a plan thread takes per tile
 constexpr float kRescaleSlack = 8.0f;  // log2 units: the running max lags by at most 2^8
-constexpr int kRopeThreads = 256;
+constexpr int kRopeThreads = 384;  // at most
 
 // ------------------------------------------------------------------------------------
 // 1. plan
@@ -266,19 +266,25 @@ __device__ __forceinline__ void split_double(double x, float &hi, float &lo) {
 __device__ __forceinline__ int cs_index(int i) { return (i & ~7) | ((i + (i >> 3)) & 7); }
 
 // One block per row.  Thread t owns the eight pairs (i, i + d/2), i = 8 (t % (d/16)) .. + 7, of
-// heads t / (d/16), t / (d/16) + 256 / (d/16), ... (query heads, then key heads): a 16-byte load
-// and store of each half.  The plan left the row's position and pool row in row_info, so every
+// heads t / (d/16), t / (d/16) + threads / (d/16), ... (query heads, then key heads): a 16-byte load
+// and store of each half.  The block is as large as the row's heads ask for, up to kRopeThreads, so
+// that the usual rows take one pass (kMore: more than one): a block's time is its chain of loads and
+// one rotation, and rows in flight are what covers it.  Held at the registers of five blocks of
+// kRopeThreads (six of 320 threads are resident); the whole call of 4 x 4096 rows of 40 heads: 482 us,
+// 491 at four, 508 at three, 487 with blocks of 256 threads in two uneven passes; 2 x 4096 rows of 16
+// heads 88.6 and 96.2; 4 x 2048 rows at head_dim 64 262.8 and 270.7.  The plan left the row's position and pool row in row_info, so every
 // load the block makes needs only the row index, and is issued at once: the first two heads'
 // halves, a 16-byte piece of the value row, and then the (cos, sin) row of the position, which
 // goes to shared memory, read by the threads of every head.
-template <int D, typename OutT>
-__global__ void __launch_bounds__(kRopeThreads) prefill_rope_kernel(PrefillView v) {
-  constexpr int kHalf = D / 2, kOcts = kHalf / 8, kHeadsPass = kRopeThreads / kOcts;
+template <int D, typename OutT, bool kMore>
+__global__ void __launch_bounds__(kRopeThreads, kMore ? 3 : 5) prefill_rope_kernel(PrefillView v) {
+  constexpr int kHalf = D / 2, kOcts = kHalf / 8;
+  const int threads = blockDim.x, heads_pass = threads / kOcts;
   constexpr int kVPieces = D / 8;  // 16-byte pieces of one head's value row
   static_assert(kHalf <= kRopeThreads, "one thread a frequency");
   __shared__ float4 cs_s[kHalf];   // (c_hi, c_lo, s_hi, s_lo) of frequency i at cs_index(i)
   const int64_t r = blockIdx.x;
-  const int tid = threadIdx.x, j = tid % kOcts, h0 = tid / kOcts, h1 = h0 + kHeadsPass;
+  const int tid = threadIdx.x, j = tid % kOcts, h0 = tid / kOcts, h1 = h0 + heads_pass;
   const int Hq = v.n_q_heads, Hkv = v.n_kv_heads, H = Hq + Hkv, nv = Hkv * kVPieces;
   uint16_t *const qrow = v.q + r * Hq * D;
   const uint16_t *const krow = v.k_new + r * Hkv * D;
@@ -291,7 +297,7 @@ __global__ void __launch_bounds__(kRopeThreads) prefill_rope_kernel(PrefillView 
   //    not stored; the call's offsets are valid when sequence 0's plan entry says so)
   uint4 x0l{}, x0h{}, x1l{}, x1h{}, vv{};
   if (h0 < H) { x0l = half_of(h0, 0); x0h = half_of(h0, 1); }
-  if (h1 < H) { x1l = half_of(h1, 0); x1h = half_of(h1, 1); }
+  if (kMore && h1 < H) { x1l = half_of(h1, 0); x1h = half_of(h1, 1); }
   if (tid < nv) vv = vrow[tid];
   grid_dependency_wait();
   grid_launch_dependents();  // the attention may be scheduled as this grid drains
@@ -303,7 +309,7 @@ __global__ void __launch_bounds__(kRopeThreads) prefill_rope_kernel(PrefillView 
   if (tid < kHalf && in_table) c4 = v.rope_table_ff[(int64_t)p * kHalf + tid];
   if (!offsets_ok || ri.y < 0) {  // not stored: its output rows are 0
     OutT *o = static_cast<OutT *>(v.out) + r * Hq * D;
-    for (int e = tid; e < Hq * D; e += kRopeThreads) o[e] = OutT(0.f);
+    for (int e = tid; e < Hq * D; e += threads) o[e] = OutT(0.f);
     return;
   }
   // 2. the (cos, sin) row in shared memory (past the table: from fp64 sincos) and the slot's
@@ -331,7 +337,7 @@ __global__ void __launch_bounds__(kRopeThreads) prefill_rope_kernel(PrefillView 
   };
   // 3. the value row (a bit copy)
   if (tid < nv) reinterpret_cast<uint4 *>(pool_row(v.v_pool, tid / kVPieces))[tid % kVPieces] = vv;
-  for (int e = tid + kRopeThreads; e < nv; e += kRopeThreads)
+  for (int e = tid + threads; e < nv; e += threads)
     reinterpret_cast<uint4 *>(pool_row(v.v_pool, e / kVPieces))[e % kVPieces] = vrow[e];
   // 4. query heads in place, key heads into the slot
   // Every output by the fast path, two to a conversion; the rare outputs whose rounding the
@@ -386,9 +392,11 @@ __global__ void __launch_bounds__(kRopeThreads) prefill_rope_kernel(PrefillView 
     *reinterpret_cast<uint4 *>(dst + kHalf + 8 * j) = make_uint4(wh[0], wh[1], wh[2], wh[3]);
   };
   if (h0 < H) rotate_store(h0, x0l, x0h);
-  if (h1 < H) rotate_store(h1, x1l, x1h);
-  for (int h = h1 + kHeadsPass; h < H; h += kHeadsPass)
-    rotate_store(h, half_of(h, 0), half_of(h, 1));
+  if constexpr (kMore) {
+    if (h1 < H) rotate_store(h1, x1l, x1h);
+    for (int h = h1 + heads_pass; h < H; h += heads_pass)
+      rotate_store(h, half_of(h, 0), half_of(h, 1));
+  }
 }
 
 // ------------------------------------------------------------------------------------
@@ -1132,9 +1140,14 @@ cudaError_t launch_all(const CUtensorMap &tk, const CUtensorMap &tv, const Prefi
   prefill_plan_kernel<<<(unsigned)v.batch, kPlanThreads, 0, stream>>>(v, prefill_query_rows(G));
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  e = launch_dependent(v.head_dim == 128 ? prefill_rope_kernel<128, OutT>
-                                         : prefill_rope_kernel<64, OutT>,
-                       (unsigned)v.rows, kRopeThreads, 0, stream, v);
+  // RoPE: a thread for every eight pairs of the row's heads, in equal passes of at most kRopeThreads
+  const int octs = (v.n_q_heads + v.n_kv_heads) * (v.head_dim / 16);
+  const int passes = (octs + kRopeThreads - 1) / kRopeThreads;
+  const int threads = max(64, ((octs + passes - 1) / passes + 31) / 32 * 32);
+  const auto rope = v.head_dim == 128
+                        ? (passes > 1 ? prefill_rope_kernel<128, OutT, true> : prefill_rope_kernel<128, OutT, false>)
+                        : (passes > 1 ? prefill_rope_kernel<64, OutT, true> : prefill_rope_kernel<64, OutT, false>);
+  e = launch_dependent(rope, (unsigned)v.rows, threads, 0, stream, v);
   if (e != cudaSuccess) return e;
   return v.head_dim == 128 ? launch_attn<128, OutT>(tq, tk, tv, v, stream)
                            : launch_attn<64, OutT>(tq, tk, tv, v, stream);

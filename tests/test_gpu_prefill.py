@@ -119,6 +119,19 @@ def test_prefill_tile_edges(hq, hkv, d, cached, rows):
     assert_parity(_out(out), ref, what="prefill output")
 
 
+# The rotation's blocks: the smallest (64 threads), one pass of 288, 320 and 384, two passes, three.
+@pytest.mark.parametrize("hq,hkv,d", [(1, 1, 64), (64, 8, 64), (32, 8, 128), (24, 24, 128), (64, 8, 128),
+                                      (96, 12, 128)])
+def test_prefill_rotation_passes(hq, hkv, d):
+    w = _w(2, hq, hkv, d, 16, seed=hq + d)
+    case = wl.make_prefill_case(w, (35, 2), cached=np.array([3, 90], np.int32))
+    kv, q, out = _gpu(case)
+    oc, q_ref, rc, ref = _oracle(case)
+    assert rc == 0
+    _check_state(kv, q, oc, q_ref)
+    assert_parity(_out(out), ref, what="prefill output")
+
+
 @pytest.mark.parametrize("d", [64, 128])
 def test_prefill_rising_maximum(d):
     """Scores with a standard deviation of 16: the running maximum rises past 2^8 in many rows after
