@@ -1202,8 +1202,9 @@ inline bool combine_early(const AttnView &v, int64_t combine_ctas, bool step) {
 // Early mode's merge: a segment spans about ctas / segments + 1 CTAs when the lengths are equal.
 // From 24 partials a segment on, a block of 64 pairs shares them among kCombineSplit groups of
 // threads (33 partials, one sequence of 2048 slots: 8.5 us a step against 10.6 with one thread reading
-// 32 at a time), as long as these smaller blocks still sit beside the pass; 16 in flight save round
-// trips from 7 on.
+// 32 at a time), as long as these smaller blocks still sit beside the pass.  From 7 on two
+// groups read 8 each (8 x 2048 slots 16.0 us a step, 8 x 4096 25.1; one thread reading 16 at a time
+// 16.9 and 25.4; two groups of 6 16.2 and 25.2).
 template <typename OutT, bool kStep>
 cudaError_t launch_combine(const AttnView &v, int head_dim, cudaStream_t stream) {
   const int pairs = v.group * head_dim / 2;
@@ -1227,9 +1228,11 @@ cudaError_t launch_combine(const AttnView &v, int head_dim, cudaStream_t stream)
   cfg.gridDim = dim3((unsigned)(segs * per_seg));
   if (!combine_early(v, segs * per_seg, kStep))
     return cudaLaunchKernelEx(&cfg, combine_late_kernel<OutT, kStep>, v, head_dim, per_seg);
-  if ((int64_t)v.ctas >= 7 * segs)
-    return cudaLaunchKernelEx(&cfg, combine_kernel<OutT, kStep, 16, kCombineThreads, 1>, v, head_dim,
+  if ((int64_t)v.ctas >= 7 * segs) {
+    cfg.blockDim = dim3(2 * kCombineThreads);
+    return cudaLaunchKernelEx(&cfg, combine_kernel<OutT, kStep, 8, kCombineThreads, 2>, v, head_dim,
                               per_seg);
+  }
   return cudaLaunchKernelEx(&cfg, combine_kernel<OutT, kStep, 8, kCombineThreads, 1>, v, head_dim,
                             per_seg);
 }

@@ -165,6 +165,28 @@ def test_step_split_counts(ctas):
     _assert_cache_equal(kv, oc)
 
 
+@pytest.mark.parametrize("d,hkv,ctas", [(128, 4, 84), (128, 4, 300), (64, 8, 120), (64, 8, 190)])
+def test_step_two_group_merge(d, hkv, ctas):
+    """7 to 24 CTAs a segment: two groups of threads share a segment's partials, of which there are
+    none, one, up to one batch a group, and more."""
+    counts = (0, 16, 333)
+    case = small_case(batch=3, hq=4 * hkv, hkv=hkv, d=d, page=16, counts=counts, seed=d + ctas,
+                      extra_slots=4)
+    big = small_case(batch=1, hq=4 * hkv, hkv=hkv, d=d, page=16, counts=(2900,), seed=ctas,
+                     extra_slots=4)
+    for c, n in ((case, ctas), (big, 8 * hkv), (big, 23 * hkv)):
+        oc = oracle.OracleCache.from_case(c)
+        kv = gpu_cache(c)
+        ham.ham_kv_set_attn_ctas(kv, n)
+        assert_parity(gpu_decode(kv, c.q, f32=True), oc.decode_attn(c.q), what="attention")
+        q_ref = c.q.copy()
+        assert oc.append(c.k_new, c.v_new, c.ntok_new, q_inout=q_ref) == 0
+        got, q_rot = _step(kv, c.q, c.k_new, c.v_new, c.ntok_new)
+        assert np.array_equal(q_rot, q_ref)
+        assert_parity(got, oc.decode_attn(q_ref), what="step")
+        _assert_cache_equal(kv, oc)
+
+
 @pytest.mark.parametrize("given", [False, True])
 @pytest.mark.parametrize("ctas", [1, 3])
 @pytest.mark.parametrize("d", [64, 128])
