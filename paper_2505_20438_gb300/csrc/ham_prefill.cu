@@ -54,6 +54,7 @@
 #include "ham_internal.cuh"
 #include "ham_prefill.cuh"
 #include "ham_ptx.cuh"
+#include "ham_turns.cuh"
 
 namespace ham {
 namespace {
@@ -857,11 +858,12 @@ __global__ void __launch_bounds__(TcShape<D>::kThreads, 1)
     const uint32_t t_s = tmem + lane_base + q * S::kTile;  // the two blocks of S_q, then P_q
     const uint32_t t_o = tmem + lane_base + S::kOffO + q * D;
     const float sl2 = (float)(1.4426950408889634 / sqrt((double)D));  // 1/sqrt(d), log2(e)
-    uint32_t sp = 0, np = 0, oc = 0, turns = 0;  // phase parities of s_full; blocks, items, turns so far
+    // phase parities of s_full; blocks, items and turns so far
+    uint32_t sp = 0, np = 0, oc = 0, turns = turns_before(q);
     bool ok = true;
     for (uint32_t k = 0;; ++k) {
       int tbase, tend, lim, lim_min;  // first slot of the block, of the item's end; row limits
-      int take_lo, take_hi, give_hi;  // tiles (first slots) that take and give the turn
+      int turn_end;                   // the blocks before this slot belong to tiles that take turns
       int64_t orow = -1;              // the row's place in out (or in the split's partials)
       bool whole;
       {
@@ -875,12 +877,9 @@ __global__ void __launch_bounds__(TcShape<D>::kThreads, 1)
         tbase = it.t0 * S::kTile;
         tend = min(tbase + nt * S::kTile, q ? it.end1 : it.end0);
         whole = it.zs == 1;
-        // Turns, in the tiles that both Q tiles read: Q tile 1's softmax of a tile follows Q tile 0's,
-        // which follows Q tile 1's of the tile before.
-        const int both = it.nt1 > 0 ? tbase + it.nt0 * S::kTile : tbase;  // end of those tiles
-        take_lo = tbase + (q == 0 ? S::kTile : 0);
-        take_hi = both;
-        give_hi = both - (q == 0 ? 0 : S::kTile);
+        // Q tile 1's softmax of a tile that both read follows Q tile 0's, which follows Q tile 1's of
+        // the shared tile before, in this item or an earlier one.
+        turn_end = tbase + turn_tiles(it.nt0, it.nt1) * S::kTile;
         if (j < it.n)
           orow = ((whole ? 0 : (int64_t)it.z * v.rows) + it.row0 + j) * Hq + it.g * G + m % G;
       }
@@ -892,7 +891,7 @@ __global__ void __launch_bounds__(TcShape<D>::kThreads, 1)
             break;
           }
           sp ^= 1u << buf;
-          if (S::kTileS && tbase >= take_lo && tbase < take_hi) {
+          if (S::kTileS && tbase < turn_end) {
             if (!warp_wait_small(&turn[q], turns & 1u, abort_flag, wait_lim)) {
               ok = false;
               break;
@@ -952,8 +951,8 @@ __global__ void __launch_bounds__(TcShape<D>::kThreads, 1)
             pk[c / 2] = pack_bf16x2(p0, p1);
             pk[c / 2 + 1] = pack_bf16x2(p2, p3);
           }
-          if (x == 1 && S::kTileS && (buf == 1 || tbase + S::kBlock >= tend) &&
-              tbase - (int)buf * S::kBlock < give_hi && lane == 0)
+          if (x == 1 && S::kTileS && tbase < turn_end && (buf == 1 || tbase + S::kBlock >= tend) &&
+              lane == 0)
             mbar_arrive(&turn[q ^ 1]);
           tmem_st16(t_b + 16 * x, pk);  // 32 probabilities as 16 bf16 pairs
         }
