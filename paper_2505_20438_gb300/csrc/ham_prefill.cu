@@ -732,8 +732,12 @@ __global__ void __launch_bounds__(TcShape<D>::kThreads, 1)
       // The first S of an item (two where S goes by blocks), then block by block O += P V once the
       // softmax group has written P, and the S whose columns are free then.  What holds an item's
       // end takes only the 16-slot chunks it reaches (N of S, K of P V).  Both warps release every
-      // K and V stage: by a commit after the products that read it, or by an arrival where their Q
-      // tile has none, so that neither falls a ring's turn behind.  Everything the products'
+      // K and V stage by a commit, also where their Q tile has no product: commits complete in the
+      // order of issue, so a warp releases the ring's stages in their order (but for a tile's V and the
+      // next tile's K, which change places).  The producers need that: a stage of an odd ring is
+      // filled by the two in turn, and a producer that waits, by parity, for the other's fill to be
+      // released relies on the fill before that one having been released too, which follows from the
+      // release its own last entry waited for, five entries earlier.  Everything the products'
       // operands depend on is kept uniform over the warp: with per-thread values an issue took
       // about 100 cycles, against the 32 to 64 that the product itself takes.
       constexpr uint32_t id_o = idesc_bf16(128, D, true);  // P from TMEM, MN-major V
@@ -838,7 +842,8 @@ __global__ void __launch_bounds__(TcShape<D>::kThreads, 1)
         }
         for (uint32_t x = e0 + 2 * nt; ok && x != e; ++x) {  // tiles it does not reach
           ok = wait_entry(x);
-          if (ok && lane == 0) mbar_arrive(&empty[x % S::kStages]);
+          if (ok && elect_one()) tc_commit(&empty[x % S::kStages]);
+          __syncwarp();
         }
       }
       if (!ok) give_up();

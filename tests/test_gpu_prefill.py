@@ -119,6 +119,30 @@ def test_prefill_tile_edges(hq, hkv, d, cached, rows):
     assert_parity(_out(out), ref, what="prefill output")
 
 
+# Many short chunks of unequal length: a CTA runs many items of one tile and a few of several, with
+# and without rows for its second Q tile, one after the other (at least six a CTA).
+@pytest.mark.parametrize("f32", [False, True])
+@pytest.mark.parametrize("hq,hkv,d,batch,longest,cached", [
+    (8, 8, 128, 150, 256, 130),      # group 1: 128-row Q tiles
+    (16, 8, 128, 130, 140, 130),     # group 2
+    (32, 8, 128, 130, 70, 130),      # group 4: one or two items a sequence
+    (32, 8, 128, 128, 64, 400),      # up to four tiles an item
+    (32, 8, 64, 130, 70, 130),
+    (16, 8, 64, 130, 140, 400),
+])
+def test_prefill_many_short_chunks(hq, hkv, d, batch, longest, cached, f32):
+    w = _w(batch, hq, hkv, d, 16, seed=hq + longest + cached)
+    rng = wl.rng_for(hq + d, longest + cached)
+    rows = tuple(int(x) for x in rng.integers(0, longest + 1, batch))
+    case = wl.make_prefill_case(w, rows, cached=rng.integers(0, cached + 1, batch).astype(np.int32))
+    kv, q, out = _gpu(case, f32=f32)
+    oc, q_ref, rc, ref = _oracle(case)
+    assert rc == 0
+    assert ham.ham_kv_status(kv) == ham.HAM_DEVERR_NONE
+    _check_state(kv, q, oc, q_ref)
+    assert_parity(_out(out), ref, what="prefill output")
+
+
 # The rotation's blocks: the smallest (64 threads), one pass of 288, 320 and 384, two passes, three.
 @pytest.mark.parametrize("hq,hkv,d", [(1, 1, 64), (64, 8, 64), (32, 8, 128), (24, 24, 128), (64, 8, 128),
                                       (96, 12, 128)])

@@ -60,6 +60,8 @@ class Cta:
     """One run.  Roles are generators that yield (barrier, phase) to wait for; phase n is the n-th
     completion, seen by the parity of n as the kernel sees it."""
 
+    in_order = True  # a tile without products is released behind the products before it
+
     def __init__(self, items, rule, stages, tile_s, seed):
         (self.turns, self.before), self.items = rule, items
         self.rng, self.tile_s, self.stages = random.Random(seed), tile_s, stages
@@ -154,7 +156,10 @@ class Cta:
                     pipe.append(self.empty[ev % self.stages])
             for x in range(e0 + 2 * nt, e):
                 yield entry(x)
-                self.empty[x % self.stages].arrive()
+                if self.in_order:
+                    pipe.append(self.empty[x % self.stages])
+                else:
+                    self.empty[x % self.stages].arrive()
 
     def softmax(self, q):
         seen, done, outs, turns = [0, 0], 0, 0, self.before[q]
@@ -222,7 +227,8 @@ def _items(rng, kinds):
     return [(*rng.choice(kinds), rng.randrange(4)) for _ in range(rng.randint(3, 9))]
 
 
-RUNS = [[(1, 1)], [(1, 2)], [(1, 0), (1, 1)], [(1, 1), (1, 2), (2, 2)], [(4, 5), (1, 1), (1, 2)]]
+RUNS = [[(1, 1)], [(1, 2)], [(1, 0), (1, 1)], [(1, 1), (1, 2), (2, 2)], [(4, 5), (1, 1), (1, 2)],
+        [(1, 0), (1, 2), (2, 3), (3, 3)], [(1, 0), (4, 5)], [(1, 0), (4, 0), (3, 3)]]
 
 
 @pytest.mark.parametrize("kinds", RUNS)
@@ -239,3 +245,15 @@ def test_turns_within_items_only_are_found_out():
     wrong = {Cta(_items(rng, [(1, 1), (1, 2)]), (within_items, [0, 0]), 5, True, seed).run()
              for seed in range(200)}
     assert "a barrier is two phases ahead of a wait" in wrong
+
+
+def test_releases_out_of_order_are_found_out(rule):
+    """Stages of tiles that a Q tile does not reach, released ahead of the products before them: a
+    producer can find a stage free that is still read."""
+    rng = random.Random(1)
+    wrong = set()
+    for seed in range(400):
+        cta = Cta(_items(rng, [(1, 0), (1, 2), (2, 3), (3, 3)]), rule, 5, True, seed)
+        cta.in_order = False
+        wrong.add(cta.run())
+    assert "a wait ends before its phase" in wrong
