@@ -22,8 +22,9 @@
 //     the call's tokens) gives zeros and sets the error word.
 // Every launch is a programmatic dependent launch of the one before (the next call's
 // projection included): it is scheduled while its predecessor runs, reads only inputs and
-// weights until its dependency wait, and waits before the first read of what the predecessor
-// wrote; the four are a chain of short latency-bound steps, so the overlap is most of the gain.
+// weights until its dependency wait, writes nothing before it, and does not end without it (in at
+// least one thread), so that a wait always covers everything before it on the stream; the four are a
+// chain of short latency-bound steps, so the overlap is most of the gain.
 // The weights (4 H^2 bf16) dominate the bytes of a call: memory-bound at decoding batches,
 // where the token rows are far fewer than the weight rows.
 // With token ids (ham_embed_tokens) step 1 is a lookup: the projections of every vocabulary
@@ -91,8 +92,10 @@ __global__ void __launch_bounds__(256) fuse_kernel(const float *__restrict__ qkv
   // the output projection may be scheduled now: it reads only its weights until its dependency
   // wait, which waits for this whole grid
   grid_launch_dependents();
-  // launched dependent on the Q/K/V projection: everything before the wait reads only the call's
-  // inputs and the handle's tables; the wait precedes the first read of its parts
+  // Everything before the dependency wait reads only the call's inputs and the handle's tables, and
+  // nothing is written before it.  A warp without a patch ends at once (its block's place goes to one
+  // that has; with every warp waiting the call took 24.3 us, not 23.5), but warp 0 waits in any case, so
+  // that the grid's end means the end of everything before it on the stream.
   const int warp = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
   const int lane = threadIdx.x & 31;
   if (warp >= batch * n_heads) return;
@@ -112,15 +115,16 @@ __global__ void __launch_bounds__(256) fuse_kernel(const float *__restrict__ qkv
   }
   __nv_bfloat16 *orow = o + (int64_t)b * H + (int64_t)h * hd;
   __nv_bfloat16 *lorow = o_lo + (int64_t)b * H + (int64_t)h * hd;
-  if (bad || n == 1) {  // the finish kernel handles these rows; O is not used for them
+  if (bad || n == 1) {  // the finish kernel handles these rows; what o holds for them is not used
     if (bad && h == 0 && lane == 0) record_error(err, HAM_DEVERR_NTOK);
-#pragma unroll
-    for (int e = 0; e < kPer; ++e) orow[lane + 32 * e] = lorow[lane + 32 * e] = __float2bfloat16_rn(0.f);
+    constexpr int kLines = (kPer * 64 + 127) / 128;
+    if (lane < 2 * kLines)  // (the projection reads them all the same: 23.9 us without)
+      asm volatile("prefetch.global.L2 [%0];" ::"l"((lane & 1 ? lorow : orow) + (lane >> 1) * 64));
+    if (warp == 0) grid_dependency_wait();
     return;
   }
   const int64_t ld = 3 * (int64_t)H, part = (int64_t)total * ld;
   const int64_t col = (int64_t)h * hd + lane;
-  const bool tabulated = ids != nullptr;  // the tables were written when the handle was made
   // the patch's loads a round trip at a time: the position terms, then each part's q, k and v
   // rows of every token at once (the parts are added in their order)
   float qv[kMaxPatch][kPer], kv[kMaxPatch][kPer], vv[kMaxPatch][kPer];
@@ -135,7 +139,7 @@ __global__ void __launch_bounds__(256) fuse_kernel(const float *__restrict__ qkv
       vv[i][e] = in ? pp[H + 32 * e] : 0.f;
     }
   }
-  if (!tabulated) grid_dependency_wait();
+  grid_dependency_wait();
   for (int sp = 0; sp < nparts; ++sp) {
     const float *base = qkv + sp * part + col;
 #pragma unroll
@@ -207,11 +211,14 @@ __global__ void finish_kernel(const float *__restrict__ part, int nparts,
                               int H, int max_patch) {
   // the next call's projection may be scheduled now (it waits for this grid before its first
   // read of anything a call writes); launched dependent on the output projection, this kernel
-  // reads the call's inputs first and waits before the first read of the parts
+  // reads the offsets and ids first; every thread waits before it reads anything else, writes or ends
   grid_launch_dependents();
   const int b = blockIdx.y;
   const int j = 8 * (blockIdx.x * blockDim.x + threadIdx.x);
-  if (b >= batch || j >= H) return;
+  if (b >= batch || j >= H) {
+    grid_dependency_wait();
+    return;
+  }
   const int t0 = offsets[b], n = offsets[b + 1] - t0;
   bool bad = n < 1 || n > max_patch || t0 < 0 || t0 + n > total;
   int xrow = t0;
@@ -223,10 +230,12 @@ __global__ void finish_kernel(const float *__restrict__ part, int nparts,
     }
   }
   uint4 v = make_uint4(0, 0, 0, 0);
+  // (x is read after the wait too, its rows may be the states of an earlier call; into L2 before it)
+  if (!bad && n == 1) asm volatile("prefetch.global.L2 [%0];" ::"l"(x + (int64_t)xrow * H + j));
+  grid_dependency_wait();
   if (!bad && n == 1) {
     v = *reinterpret_cast<const uint4 *>(x + (int64_t)xrow * H + j);
   } else if (!bad) {
-    grid_dependency_wait();
     // the parts added in their order, loaded kBatch at a time (one round trip each batch)
     constexpr int kBatch = 10;
     float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};

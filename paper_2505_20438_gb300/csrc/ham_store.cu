@@ -114,16 +114,27 @@ int fp8_unsupported(const ham_kv *kv, const char *call) {
 }
 
 // ---------------------------------------------------------------------------------------
-// Early start.  The attention kernels are launched with programmatic dependent launch and can
-// read their layer's counters, page table and pools before their dependency wait, which lets
-// the plan and the first K/V copies overlap the previous kernel, provided that kernel does not
-// write them.  Every kernel of this library waits for its own predecessor before letting its
-// successor start, so when an attention grid starts, everything before the immediately
-// preceding kernel has completed; only that kernel may still run.  The library remembers, per
-// stream (and per stream capture), the last launch it made and which (handle, layer) state it
-// writes, and allows the early start only when that launch is known and leaves this layer
-// alone.  Kernels of other code in between are harmless: they cannot write a handle's state
-// (only these calls do), and an unknown predecessor means no early start.
+// Early start.  The attention and micro-step kernels are launched with programmatic dependent launch
+// and can read their layer's counters, page table and pools before their dependency wait, which lets
+// the plan and the first K/V copies overlap the kernels before, provided none of these that still run
+// writes them.  Two properties of the library's kernels bound what may still run:
+//  - No grid ends without a dependency wait in at least one of its threads, or it was launched in
+//    full stream order.  So a wait covers everything before it on the stream, not only the kernel
+//    before.  Nothing is written before the wait but by the combine (q_rot, the new slot's rows, its
+//    arrival count), which starts after its own pass has waited: only that pass may still run, and it
+//    touches none of these.
+//  - Several kernels let their successor start before their own wait (the combine; the embedder's
+//    projections, fusion and finish), so a kernel may start while several before it still run.  But
+//    the first kernel of every call noted below lets its successor start only after its own wait, or
+//    was launched in full stream order (the prefill's plan, the fills, set_lengths).  What comes after
+//    it on the stream starts only when everything before that call has completed: of the noted calls
+//    only the last one may still run.
+// That call writes only its layer's state, its outputs and its handle's scratch, which a following
+// kernel touches after its wait; calls that are not noted (the embedder, ham_decode_attn_noalloc)
+// write no handle's state.  The library remembers, per stream (and per stream capture), the last noted
+// call and which (handle, layer) state it writes, and allows the early start only when that call is
+// known and leaves this layer alone.  Kernels of other code in between are harmless: they cannot write
+// a handle's state (only these calls do), and an unknown predecessor means no early start.
 // ---------------------------------------------------------------------------------------
 struct LastLaunch {
   const ham_kv *kv;

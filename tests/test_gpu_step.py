@@ -342,3 +342,92 @@ def test_step_full_size(w):
     assert_parity(got, ref, what=w.name)
     # the appended rows, bit for bit (the whole pool at this size is compared too)
     _assert_cache_equal(kv, oc)
+
+
+@pytest.mark.parametrize("seed", range(4))
+def test_calls_back_to_back(seed):
+    """Steps, micro-steps, the two separate calls, prefills and the embedder (sequences of one token
+    and of several, token ids and rows, states of one call as rows of the next) on one stream with
+    nothing between them: the bits of the same calls with a synchronisation after each."""
+    t = torch()
+    d, hq, hkv, B = 64, 8, 2, 4
+    small = small_case(batch=B, hq=hq, hkv=hkv, d=d, page=16, counts=(0, 1, 3, 5), seed=seed, extra_slots=11)
+    large = small_case(batch=B, hq=hq, hkv=hkv, d=d, page=16, counts=(300, 17, 0, 64), seed=seed + 9,
+                       extra_slots=160)
+    ew = wl.embed_workload(B, hidden=256, n_heads=8, seed=seed)
+    tc = wl.make_embed_tokens_case(ew, 500)
+    c = tc.case
+    g = t.Generator(device="cuda")
+    g.manual_seed(seed)
+
+    def normal(*shape):
+        return t.randn(shape, generator=g, device="cuda").to(t.bfloat16)
+
+    rng = wl.rng_for(seed, 40)
+    calls = []
+    for i in range(120):
+        kind = ("step", "micro", "lone", "split", "tokens", "step", "chain", "embed", "prefill")[rng.integers(9)]
+        rows = 5 * B if kind == "prefill" else B
+        calls.append((kind, int(rng.integers(3)), normal(rows, hq, d), normal(rows, hkv, d), normal(rows, hkv, d)))
+    ones = dev_i32(np.ones(B))
+    lone = dev_i32(np.arange(B + 1))
+    pairs = dev_i32(np.array([0, 2, 4]))
+    chunks = dev_i32(5 * np.arange(B + 1))
+    ids, x, offsets = dev_i32(tc.ids), dev_bf16(c.x), dev_i32(c.offsets)
+    lone_ids = dev_i32(tc.ids[:B])
+    start = [dev_i32(case.num_slots) for case in (small, large)]
+
+    def run(wait):
+        kvs = [gpu_cache(small, layers=3), gpu_cache(large, layers=3)]
+        e = ham.ham_embedder_alloc(ew.hidden, ew.n_heads, B, ew.max_patch, dev_bf16(c.wq), dev_bf16(c.wk),
+                                   dev_bf16(c.wv), dev_bf16(c.wo), dev_bf16(c.pos))
+        ham.ham_embedder_set_vocab(e, dev_bf16(tc.table))
+        bufs = [(q.clone(), t.zeros_like(q), t.zeros_like(q)) for _, _, q, _, _ in calls]
+        states = [t.zeros((B, ew.hidden), dtype=t.bfloat16, device="cuda") for _ in range(len(calls) + 1)]
+        used = [[0] * 3, [0] * 3]
+        t.cuda.synchronize()
+        for i, (kind, layer, _, k, v) in enumerate(calls):
+            q, out, q_rot = bufs[i]
+            which = 0 if kind == "micro" or (kind in ("step", "split") and i % 2) else 1
+            if kind not in ("lone", "tokens", "chain", "embed"):
+                used[which][layer] += 5 if kind == "prefill" else 1
+                if used[which][layer] > (9, 150)[which]:  # drop what this run appended
+                    ham.ham_kv_set_lengths(kvs[which], layer, start[which])
+                    used[which][layer] = 5 if kind == "prefill" else 1
+            kv = kvs[which]
+            if kind == "step":
+                ham.ham_decode_step(kv, layer, q, k, v, None, ones, out, q_rot=q_rot)
+            elif kind == "micro":
+                ham.ham_micro_step(kv, layer, q, k, v, None, ones, out, q_rot=q_rot)
+            elif kind == "split":
+                ham.ham_kv_append(kv, layer, q, k, v, None, ones)
+                ham.ham_decode_attn_ex(kv, layer, q, out)
+            elif kind == "prefill":
+                ham.ham_prefill(kv, layer, q, k, v, chunks, out)
+            elif kind == "lone":
+                ham.ham_embed_tokens(e, lone_ids, lone, states[i + 1])
+            elif kind == "tokens":
+                ham.ham_embed_tokens(e, ids, offsets, states[i + 1])
+            elif kind == "chain" and i % 2:  # the newest states as the rows
+                ham.ham_embed(e, states[i], lone, states[i + 1])
+            elif kind == "chain":
+                ham.ham_embed(e, states[i], pairs, states[i + 1][:2])
+            else:
+                ham.ham_embed(e, x, offsets, states[i + 1])
+            if kind not in ("lone", "tokens", "chain", "embed"):
+                states[i + 1] = states[i]
+            if wait:
+                t.cuda.synchronize()
+        t.cuda.synchronize()
+        got = [host_bits(y) for b in bufs for y in b] + [host_bits(y) for y in states]
+        for kv in kvs:
+            for layer in range(3):
+                got += list(_export_host(kv, layer)) + list(ham.ham_kv_layer_lengths(kv, layer))
+            assert ham.ham_kv_status(kv) == ham.HAM_DEVERR_NONE
+        assert ham.ham_embedder_status(e) == ham.HAM_DEVERR_NONE
+        return got
+
+    want = run(True)
+    for _ in range(3):
+        for a, b in zip(want, run(False)):
+            assert np.array_equal(a, b)
