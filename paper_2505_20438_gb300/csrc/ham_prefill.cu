@@ -11,8 +11,8 @@
 // Three launches (four when the attention splits over the cached slots):
 //  1. prefill_plan_kernel, one block per sequence: checks that the sequence's rows fit
 //     (counts, capacity, pages), gives each row its position (slot index, running token count
-//     or the caller's) and pool row (or -1: not stored), numbers the query blocks, and advances
-//     the counters.
+//     or the caller's) and pool row (or -1: not stored), orders the query blocks, and advances the
+//     token count.
 //  2. prefill_rope_kernel, one block per row: turns q and k at the row's position and stores
 //     k and v into the row's slot.  The rotation x0 c - x1 s is evaluated from the fp64 cos/sin
 //     table in pairs of fp32 values (error-free products and sums, about 48 bits) and rounded
@@ -30,7 +30,7 @@
 //     raised only past 2^8), write the bf16 probabilities over the scores (the A operand of
 //     O += P V) and rescale O in tensor memory when the maximum moves.  The causal mask applies to
 //     the blocks that reach past a row's own slot; items are handed out from a counter in the
-//     plan's order, the longest rows of the causal triangle first.
+//     plan's order, the blocks that attend over the most slots first.
 //     When the items would leave SMs idle (a short chunk: few query blocks) they are split over
 //     slots: a sequence with L cached slots is cut into up to floor(L / 512) contiguous ranges
 //     of 128-slot tiles (the last range also takes the chunk's own slots), and a split that is
@@ -52,6 +52,7 @@
 #include <type_traits>
 
 #include "ham_internal.cuh"
+#include "ham_order.cuh"
 #include "ham_prefill.cuh"
 #include "ham_ptx.cuh"
 #include "ham_turns.cuh"
@@ -98,7 +99,7 @@ __device__ __forceinline__ int block_scan(int x, int *red, int *total) {
   return x + before;
 }
 
-__global__ void __launch_bounds__(kPlanThreads) prefill_plan_kernel(PrefillView v, int qb_rows) {
+__global__ void __launch_bounds__(kPlanThreads) prefill_plan_kernel(PrefillView v, int qb_shift) {
   __shared__ int red[kPlanThreads / 32];
   const int b = blockIdx.x, tid = threadIdx.x, B = v.batch;
   // The RoPE kernel may be scheduled now: it reads the call's inputs, and waits for this grid (which
@@ -121,25 +122,34 @@ __global__ void __launch_bounds__(kPlanThreads) prefill_plan_kernel(PrefillView 
     return;
   }
   const int a = v.offsets[b], n = v.offsets[b + 1] - a;
-  // The order of the query blocks in the attention: later blocks of the chunks (longer rows of the
-  // causal triangle) first, sequence by sequence.  Block j comes after all blocks j' > j and the
-  // blocks j of earlier sequences.
-  auto blocks_of = [&](int c) { return (v.offsets[c + 1] - v.offsets[c] + qb_rows - 1) / qb_rows; };
-  for (int j = tid; j < blocks_of(b); j += kPlanThreads) {
-    int at = 0;
-    for (int c = 0; c < B; ++c) {
-      const int m = blocks_of(c);
-      at += max(0, m - 1 - j) + (c < b && m > j ? 1 : 0);
+  const int L = v.num_slots[b];
+  // The order of the query blocks in the attention (ham_order.cuh): the place of each of this
+  // sequence's, by a group of 2^g threads that share the other sequences.  The counters do not change
+  // while the plan runs: the attention, which starts after all of it, advances num_slots.
+  auto slots_of = [&](int c) { return (uint32_t)max(0, min(v.num_slots[c], v.max_slots)); };
+  {
+    const int g = B >= 32 ? 5 : 32 - __clz(B - 1);  // (B = 1: 0)
+    const int m = (int)query_blocks(n, qb_shift), share = tid & ((1 << g) - 1);
+    const uint32_t own = slots_of(b);
+    for (int j0 = 0; j0 < m; j0 += kPlanThreads >> g) {  // (the same trip count in every thread)
+      const int j = j0 + (tid >> g);
+      const uint32_t reach = block_reach(own, n, j, qb_shift);
+      uint32_t at = 0;
+      if (j < m) {
+        for (int c = share; c < B; c += 1 << g)
+          if (c != b)
+            at += blocks_before(slots_of(c), v.offsets[c + 1] - v.offsets[c], reach, c < b, qb_shift);
+      }
+      for (int o = 1; o < 1 << g; o <<= 1) at += __shfl_xor_sync(kFull, at, o);
+      if (j < m && share == 0) v.order[at + (m - 1 - j)] = make_int2(b, j);
     }
-    v.order[at] = make_int2(b, j);
   }
   if (b == 0) {
     int m = 0;
-    for (int c = tid; c < B; c += kPlanThreads) m += blocks_of(c);
+    for (int c = tid; c < B; c += kPlanThreads) m += query_blocks(v.offsets[c + 1] - v.offsets[c], qb_shift);
     m = block_sum(m, red);
     if (tid == 0) v.next_item[1] = m;
   }
-  const int L = v.num_slots[b];
   int err = 0;
   if (L < 0 || L > v.max_slots) err = HAM_DEVERR_SLOTS;
   else if ((int64_t)L + n > v.max_slots) err = HAM_DEVERR_CAPACITY;
@@ -161,7 +171,7 @@ __global__ void __launch_bounds__(kPlanThreads) prefill_plan_kernel(PrefillView 
     for (int j = tid; j < n; j += kPlanThreads) v.row_info[a + j] = make_int2(0, -1);
     if (tid == 0) {
       record_error(v.err, err);
-      v.seq_info[b] = make_int4(-1, n, 0, 1);
+      v.seq_info[b] = make_int4(-1, n, a, 1);
     }
     return;
   }
@@ -198,8 +208,7 @@ __global__ void __launch_bounds__(kPlanThreads) prefill_plan_kernel(PrefillView 
     carry += total;
   }
   if (tid == 0) {
-    v.seq_info[b] = make_int4(L, n, 0, 1);
-    v.num_slots[b] = L + n;
+    v.seq_info[b] = make_int4(L, n, a, 1);
     v.num_tokens[b] = t0 + carry;
   }
 }
@@ -405,8 +414,8 @@ __global__ void __launch_bounds__(kRopeThreads, kMore ? 3 : 5) prefill_rope_kern
 // ------------------------------------------------------------------------------------
 // A work item is one KV head, two Q tiles of 128 rows each and (split launches) one range of
 // slots; a row is a (query row, head) pair, m = (row - first row of the tile) * G + head within
-// the group, and sits in TMEM lane m.  CTAs (one an SM) take items from a counter, the longest
-// rows of the causal triangle first; an item's last softmax and output run beside the next one's
+// the group, and sits in TMEM lane m.  CTAs (one an SM) take items from a counter, the blocks that
+// attend over the most slots first; an item's last softmax and output run beside the next one's
 // first copies.
 //
 // K and V come in tiles of 128 slots; the softmax works on blocks of 64 (half tiles).  Tensor-memory
@@ -525,7 +534,7 @@ __device__ __forceinline__ bool decode_item(const PrefillView &v, int id, int nb
   it.L = L;
   it.n = n;
   it.qb0 = qb0;
-  it.row0 = v.offsets[blk.x];
+  it.row0 = si.z;
   it.z = z;
   it.zs = zs;
   it.t0 = t0;
@@ -594,6 +603,12 @@ __global__ void __launch_bounds__(TcShape<D>::kThreads, 1)
   const uint32_t tmem = *tmem_slot;
   grid_dependency_wait();  // the plan, the rotated queries and the stored rows
   grid_launch_dependents();
+  if (blockIdx.x == 0 && warp < S::kProducerWarp) {  // the slot counters (the plan's blocks read them all)
+    for (int b = tid; b < v.batch; b += S::kProducerWarp * 32) {
+      const int4 si = v.seq_info[b];
+      if (si.x >= 0) v.num_slots[b] = si.x + si.y;
+    }
+  }
   // ring and data waits: the launch's limit; item hand-over and the draining of in-flight work
   // keep the default 2 s
   const uint64_t wait_lim = data_wait_limit(v.wait_ns);
@@ -1141,7 +1156,9 @@ cudaError_t launch_all(const CUtensorMap &tk, const CUtensorMap &tv, const Prefi
   CUtensorMap tq;  // the chunk's queries, rotated in place by the RoPE kernel
   if (make_rows_tensor_map(&tq, v.q, v.rows, v.n_q_heads, v.head_dim, G, 128 / G) != 0)
     return cudaErrorInvalidValue;
-  prefill_plan_kernel<<<(unsigned)v.batch, kPlanThreads, 0, stream>>>(v, prefill_query_rows(G));
+  int qb_shift = 0;  // (a power of two)
+  while (1 << qb_shift < prefill_query_rows(G)) ++qb_shift;
+  prefill_plan_kernel<<<(unsigned)v.batch, kPlanThreads, 0, stream>>>(v, qb_shift);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   // RoPE: a thread for every eight pairs of the row's heads, in equal passes of at most kRopeThreads

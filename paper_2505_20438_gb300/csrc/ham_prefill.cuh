@@ -21,8 +21,8 @@ struct PrefillView {
   const uint16_t *k_new, *v_new;
   const int32_t *offsets, *pos, *ntok;  // pos, ntok nullable
   void *out;                   // [rows][n_q_heads][head_dim], bf16 or f32
-  int4 *seq_info;              // scratch [batch]: (first new slot or -1, rows, unused, 1 when the
-                               // call's offsets are valid, else 0)
+  int4 *seq_info;              // scratch [batch]: (first new slot or -1, rows, first row of the call,
+                               // 1 when the call's offsets are valid, else 0)
   int2 *row_info;              // scratch [rows]: (position, pool row page * page_slots + row
                                // in page, or -1 when the row is not stored) of each new row
   int32_t *err;
