@@ -650,7 +650,10 @@ constexpr int kCombineThreads = 128;
 // -2.6% (bf16) and -7% (FP8) at batch 8 x 4096 slots, -1.5% and -4% at 8192; below that
 // window it cost 2.5% (batch 1 x 16384) to 4% (8 x 200) against just before the wait, which gave
 // -10% at 8 x 200 and -9% at 1 x 300 against after it; above (batch 4 x 65536, 215 chunks a CTA)
-// either costs 1.2%, so the trigger stays after the wait there.
+// either costs 1.2%, so the trigger stays after the wait there.  So it does below the window when this
+// grid does not sit beside the pass (the attention alone, more blocks than SMs): before the wait the
+// next kernel's blocks took places that this grid's last ones were waiting for (append + attention of
+// 84 x 1500 slots, one KV head and a group of 8: 23.2 us, 22.2 after it).
 constexpr int kTriggerChunksMin = 16, kTriggerChunksMax = 128;
 constexpr int kCombineSplit = 4;  // thread groups of a block that share a segment's partials
 constexpr int kCombinePlanBatch = kCombineThreads;  // batches whose plan the combine computes
@@ -961,9 +964,10 @@ __global__ void __launch_bounds__(kPairs *kSplit) combine_kernel(const AttnView 
   }
 
   // The next kernel may be scheduled now; its own dependency wait still covers this grid.
-  if (!heavy && !lengthy) grid_launch_dependents();
+  const bool after = !heavy && (lengthy || (!kStep && gridDim.x > (unsigned)v.sms));
+  if (!heavy && !after) grid_launch_dependents();
   grid_dependency_wait();  // the attention grid's partials
-  if (lengthy) grid_launch_dependents();
+  if (after) grid_launch_dependents();
 
   const bool merge = first >= 0 && (kStep || first != last);
   float M = -INFINITY, num0 = 0.f, num1 = 0.f, den = 0.f;
@@ -1204,7 +1208,9 @@ inline bool combine_early(const AttnView &v, int64_t combine_ctas, bool step) {
 // threads (33 partials, one sequence of 2048 slots: 8.5 us a step against 10.6 with one thread reading
 // 32 at a time), as long as these smaller blocks still sit beside the pass.  From 7 on two
 // groups read 8 each (8 x 2048 slots 16.0 us a step, 8 x 4096 25.1; one thread reading 16 at a time
-// 16.9 and 25.4; two groups of 6 16.2 and 25.2).
+// 16.9 and 25.4; two groups of 6 16.2 and 25.2) while the grid has at most a block an SM: with more
+// blocks of twice the threads fewer are resident (append + attention of 42 x 300 slots, two KV heads
+// and groups of 8: 14.4 us, 13.6 with one thread reading 8).
 template <typename OutT, bool kStep>
 cudaError_t launch_combine(const AttnView &v, int head_dim, cudaStream_t stream) {
   const int pairs = v.group * head_dim / 2;
@@ -1228,7 +1234,7 @@ cudaError_t launch_combine(const AttnView &v, int head_dim, cudaStream_t stream)
   cfg.gridDim = dim3((unsigned)(segs * per_seg));
   if (!combine_early(v, segs * per_seg, kStep))
     return cudaLaunchKernelEx(&cfg, combine_late_kernel<OutT, kStep>, v, head_dim, per_seg);
-  if ((int64_t)v.ctas >= 7 * segs) {
+  if ((int64_t)v.ctas >= 7 * segs && segs * per_seg <= (int64_t)v.sms) {
     cfg.blockDim = dim3(2 * kCombineThreads);
     return cudaLaunchKernelEx(&cfg, combine_kernel<OutT, kStep, 8, kCombineThreads, 2>, v, head_dim,
                               per_seg);

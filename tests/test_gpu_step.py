@@ -187,6 +187,27 @@ def test_step_two_group_merge(d, hkv, ctas):
         _assert_cache_equal(kv, oc)
 
 
+@pytest.mark.parametrize("d,hkv,batch", [(128, 2, 42), (128, 1, 84), (64, 4, 21)])
+def test_attention_of_more_combine_blocks_than_sms(d, hkv, batch):
+    """7 to 24 CTAs a segment in groups of 8, so that the attention's combine has more blocks than SMs
+    (at head_dim 64: about as many): one thread reads all of a pair's partials, and the next call is let
+    in after the wait.  Appends and attentions in turn."""
+    rng = wl.rng_for(d, batch)
+    case = small_case(batch=batch, hq=8 * hkv, hkv=hkv, d=d, page=16,
+                      counts=tuple(int(x) for x in rng.integers(0, 700, batch)), seed=batch, extra_slots=4)
+    oc = oracle.OracleCache.from_case(case)
+    kv = gpu_cache(case)
+    assert_parity(gpu_decode(kv, case.q, f32=True), oc.decode_attn(case.q), what="attention")
+    for i in range(3):
+        q_ref, q = case.q.copy(), dev_bf16(case.q)
+        assert oc.append(case.k_new, case.v_new, case.ntok_new, q_inout=q_ref) == 0
+        out = torch().full(q.shape, float("nan"), dtype=torch().float32, device="cuda")
+        ham.ham_kv_append(kv, 0, q, dev_bf16(case.k_new), dev_bf16(case.v_new), None, dev_i32(case.ntok_new))
+        ham.ham_decode_attn_ex(kv, 0, q, out)
+        assert_parity(out.cpu().numpy().astype(np.float64), oc.decode_attn(q_ref), what=f"call {i}")
+    _assert_cache_equal(kv, oc)
+
+
 @pytest.mark.parametrize("given", [False, True])
 @pytest.mark.parametrize("ctas", [1, 3])
 @pytest.mark.parametrize("d", [64, 128])
