@@ -123,6 +123,7 @@ __global__ void __launch_bounds__(256) fuse_kernel(const float *__restrict__ qkv
     if (warp == 0) grid_dependency_wait();
     return;
   }
+  const bool tabulated = ids != nullptr;  // the tables were written when the handle was made
   const int64_t ld = 3 * (int64_t)H, part = (int64_t)total * ld;
   const int64_t col = (int64_t)h * hd + lane;
   // the patch's loads a round trip at a time: the position terms, then each part's q, k and v
@@ -139,7 +140,8 @@ __global__ void __launch_bounds__(256) fuse_kernel(const float *__restrict__ qkv
       vv[i][e] = in ? pp[H + 32 * e] : 0.f;
     }
   }
-  grid_dependency_wait();
+  // the projection's parts after the wait; tabulated rows before it, and the wait before o is written
+  if (!tabulated) grid_dependency_wait();
   for (int sp = 0; sp < nparts; ++sp) {
     const float *base = qkv + sp * part + col;
 #pragma unroll
@@ -187,6 +189,7 @@ __global__ void __launch_bounds__(256) fuse_kernel(const float *__restrict__ qkv
     den += s[i];
   }
   const float inv = 1.f / den;
+  if (tabulated) grid_dependency_wait();
 #pragma unroll
   for (int e = 0; e < kPer; ++e) {
     float acc = 0.f;
