@@ -141,10 +141,11 @@ __global__ void __launch_bounds__(kFrontThreads, NT == 1 ? 3 : 2) front_kernel(F
     const uint16_t *w_lo = v.w + ((int64_t)hh * d + p0 + gid) * H + col0;
     const uint16_t *w_hi = w_lo + (int64_t)half * H;
     // The weights are not written by kernels (a prefetch into L2 is safe in any case): pull
-    // the first columns while the previous kernel on the stream finishes: two batches of loads
-    // (12 layer fronts and attentions of batch 8, hidden 4096: 163.6 us; one batch 165.9, every
-    // column 164.9, which takes bandwidth from the kernel before).
-    for (int u = 0; u < 2 * U && u < steps; ++u) {
+    // the first columns while the previous kernel on the stream finishes: two batches of loads after
+    // an attention (4 layer fronts and attentions of batch 8, hidden 4096: 162 us; one batch 164,
+    // every column 165), one after another front, which is itself bound by the bandwidth for
+    // weights (fronts back to back 11.3 us each; two batches 12.0).
+    for (int u = 0; u < v.ahead * U && u < steps; ++u) {
       prefetch_l2(w_lo + u * 32);
       prefetch_l2(w_hi + u * 32);
     }

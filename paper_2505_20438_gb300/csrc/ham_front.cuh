@@ -40,6 +40,7 @@ struct FrontView {
   int64_t pool_pages;
   int32_t batch, hidden, n_q_heads, n_kv_heads, head_dim, page_slots, max_pages, max_slots;
   int32_t pos_mode;
+  int32_t ahead;               // batches of weight loads that are prefetched before the dependency wait
 };
 
 cudaError_t launch_front(const FrontView &v, cudaStream_t stream);

@@ -140,6 +140,7 @@ struct LastLaunch {
   const ham_kv *kv;
   int32_t layer;  // -1: every layer
   bool writes;    // wrote the layer's counters, pools or slot metadata
+  bool front;     // a layer front (ham_qkv_append), which streams weights
 };
 std::mutex g_launch_mu;
 std::map<std::pair<uintptr_t, unsigned long long>, LastLaunch> g_last_launch;
@@ -165,11 +166,18 @@ bool may_start_early(const ham_kv *kv, int32_t layer, void *stream) {
   return !(l.kv == kv && l.writes && (l.layer == layer || l.layer < 0));
 }
 
-void note_launch(const ham_kv *kv, int32_t layer, void *stream, bool writes) {
+bool last_was_front(void *stream) {
+  const auto key = launch_key(stream);
+  std::lock_guard<std::mutex> lock(g_launch_mu);
+  const auto it = g_last_launch.find(key);
+  return it != g_last_launch.end() && it->second.front;
+}
+
+void note_launch(const ham_kv *kv, int32_t layer, void *stream, bool writes, bool front = false) {
   const auto key = launch_key(stream);
   std::lock_guard<std::mutex> lock(g_launch_mu);
   if (g_last_launch.size() > 4096) g_last_launch.clear();  // forgetting is always safe
-  g_last_launch[key] = LastLaunch{kv, layer, writes};
+  g_last_launch[key] = LastLaunch{kv, layer, writes, front};
 }
 
 // Byte offsets of everything ham_kv_alloc carves out of the handle's metadata allocation (each
@@ -894,9 +902,10 @@ int ham_qkv_append(ham_kv *kv, int32_t layer, const void *x, const void *w_qkv, 
   v.max_pages = kv->max_pages;
   v.max_slots = c.max_slots_per_seq;
   v.pos_mode = c.pos_mode;
+  v.ahead = last_was_front(stream) ? 1 : 2;
   cudaError_t e = ham::launch_front(v, static_cast<cudaStream_t>(stream));
   if (e != cudaSuccess) return cuda_fail(e, "layer front launch");
-  note_launch(kv, layer, stream, true);
+  note_launch(kv, layer, stream, true, true);
   return HAM_OK;
 }
 
