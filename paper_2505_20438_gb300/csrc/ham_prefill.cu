@@ -36,10 +36,12 @@
 //     of 128-slot tiles (the last range also takes the chunk's own slots), and a split that is
 //     not alone leaves its rows' unnormalised output, running maximum and sum as a partial.
 //     Bound by each Q tile's chain scores -> softmax -> P V -> scores, which the other tile's
-//     covers in part: the tensor pipe is about 60% busy.  4 fresh prompts x 4096 rows of a
-//     Llama-8B layer, the whole call: 492 us, against 565 with 64-slot tiles, four issuing warps whose
-//     operands sat in per-thread registers and a CTA an item; 64 rows over 65,536 slots 80 against
-//     139 us (with the merge below); 4 x 2048 rows over 2048 slots at head_dim 64: 281 against 345.
+//     covers in part: the tensor pipe is about 60% busy.  The whole call, in a loop of calls on one set
+//     of buffers (with buffers that change from call to call 2% more): 4 fresh prompts x 4096 rows
+//     of a Llama-8B layer 477 us, against 565 with 64-slot tiles, four issuing warps whose operands
+//     sat in per-thread registers and a CTA an item; 64 rows over 65,536 slots 80 against 142 us (with
+//     the merge below); 4 x 2048 rows over 2048 slots at head_dim 64 263 against 345; 256 prompts of
+//     32 rows 102 against 175.
 //  4. prefill_merge_kernel (split launches only), one warp per (row, head): the split-softmax
 //     merge of the partials in split order (as the decode combine merges its CTAs').
 //
@@ -280,12 +282,13 @@ __device__ __forceinline__ int cs_index(int i) { return (i & ~7) | ((i + (i >> 3
 // and store of each half.  The block is as large as the row's heads ask for, up to kRopeThreads, so
 // that the usual rows take one pass (kMore: more than one): a block's time is its chain of loads and
 // one rotation, and rows in flight are what covers it.  Held at the registers of five blocks of
-// kRopeThreads (six of 320 threads are resident); the whole call of 4 x 4096 rows of 40 heads: 482 us,
-// 491 at four, 508 at three, 487 with blocks of 256 threads in two uneven passes; 2 x 4096 rows of 16
-// heads 88.6 and 96.2; 4 x 2048 rows at head_dim 64 262.8 and 270.7.  The plan left the row's position and pool row in row_info, so every
-// load the block makes needs only the row index, and is issued at once: the first two heads'
-// halves, a 16-byte piece of the value row, and then the (cos, sin) row of the position, which
-// goes to shared memory, read by the threads of every head.
+// kRopeThreads (six of 320 threads are resident).  The whole call in a loop, before the later changes
+// of the attention: 4 x 4096 rows of 40 heads 482 us, 491 at four, 508 at three, 487 with blocks of 256
+// threads in two uneven passes; 2 x 4096 rows of 16 heads 88.6 and 96.2; 4 x 2048 rows at head_dim 64
+// 262.8 and 270.7.  The plan left the row's position and pool row in row_info, so every load the block
+// makes needs only the row index, and is issued at once: the first two heads' halves, a 16-byte piece
+// of the value row, and then the (cos, sin) row of the position, which goes to shared memory, read by
+// the threads of every head.
 template <int D, typename OutT, bool kMore>
 __global__ void __launch_bounds__(kRopeThreads, kMore ? 3 : 5) prefill_rope_kernel(PrefillView v) {
   constexpr int kHalf = D / 2, kOcts = kHalf / 8;
@@ -422,7 +425,12 @@ __global__ void __launch_bounds__(kRopeThreads, kMore ? 3 : 5) prefill_rope_kern
 // columns per Q tile q: two blocks of scores S_q (64 fp32 each; the first 32 columns of a block then
 // hold its probabilities P, bf16 pairs, the A operand of O += P V) and O_q (head_dim fp32).  One
 // thread a Q tile issues its products: O += P V of a block, then the S whose columns that frees.
-// Products execute in issue order, so S overwrites P only after P V has read it.
+// Nothing but the order of issue says that P V has read P when S overwrites it.  PTX promises that order
+// for products on one accumulator; these two have different ones (P is an operand of the first and lies
+// in the columns that the second writes), so the kernel relies on the tensor core taking the products
+// of one thread in the order in which it issued them, whatever their accumulators.  A wait for P V before
+// S gives the same bits and costs 1 to 6% (4 x 4096 rows 507 us and 489, ragged chunks 247 and 233, 64
+// rows over 65,536 slots 81.7 and 80.6).
 //  - head_dim 128: S of a tile (N = 128) follows P V of the second block of the tile before.  While
 //    the products of one Q tile run, the other's softmax does: the two softmax groups take turns,
 //    tile by tile.  (Left to themselves they fall into step, compete for the issue slots and then

@@ -30,7 +30,7 @@ struct PrefillView {
   int32_t batch, rows, n_q_heads, n_kv_heads, head_dim, page_slots, max_pages, max_slots;
   int32_t pos_mode;
   uint64_t wait_ns;            // limit of the attention's data waits (0: the default 2 s)
-  // Split over slots (a short chunk over a long cache): the attention grid's z dimension.  A
+  // Splits over slots (a short chunk over a long cache): the slowest dimension of the work items.  A
   // sequence of L cached slots uses prefill_splits(L, splits) of them; a split that is not alone
   // leaves its rows' unnormalised partials (output, running maximum and sum) here, and the merge
   // kernel combines them: part_o [splits][rows][n_q_heads][head_dim], part_ml [same without d].
@@ -64,7 +64,7 @@ __host__ __device__ inline int prefill_splits(int L, int Z) {
   return by_len < 1 ? 1 : (by_len < Z ? by_len : Z);
 }
 // Scratch floats the split partials may use: SMs x 256 (row, head) pairs x head_dim (a launch
-// splits only while its CTAs, 256 pairs each, fit the SMs).
+// splits only into as many items, 256 pairs each, as there are SMs).
 inline size_t prefill_part_floats(int sms, int head_dim) {
   return (size_t)sms * 256 * (size_t)head_dim;
 }
